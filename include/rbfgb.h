@@ -215,7 +215,7 @@ rbf_status rbf_lm_step(rbf_ctx* ctx, const double* R, const double* t, const flo
  * of rbf_soft_cost.  Its only scratch, the per-block partial sums, lives in a
  * fixed device array of 128 KiB (2,048 blocks x 8 float64) that every GPU
  * which loads the library holds until the process exits.  The launch uses
- * min(ceil(n / 256), 4 x number of SMs) blocks, so any n is accepted on GPUs
+ * at most 4 x number of SMs blocks, so any n is accepted on GPUs
  * with up to 512 SMs; a launch that would need more blocks returns RBF_ERANGE.
  * The first call on a device looks up the array's device address
  * (cudaGetSymbolAddress) with that device current; make that first call
