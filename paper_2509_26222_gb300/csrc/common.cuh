@@ -295,8 +295,9 @@ inline cudaError_t cooperative_launch(const void* f, dim3 g, dim3 b, void** args
 constexpr int64_t BW_DENSE = BW_DENSE_CTX;
 rbf_status potrf_lower(Ctx* c, double* A, int64_t n, int64_t lda, int64_t nfactor,
                        bool mixed, cudaStream_t s, int64_t bw = BW_DENSE);
+// have_inv: the previous trsm_lower on this context was with the same L
 rbf_status trsm_lower(Ctx* c, const double* L, int64_t n, int64_t ldl, double* B, int64_t m,
-                      int64_t ldb, bool transpose, cudaStream_t s, int64_t bw = BW_DENSE);
+                      int64_t ldb, bool transpose, cudaStream_t s, int64_t bw = BW_DENSE, bool have_inv = false);
 rbf_status gemm_f64(Ctx* c, bool ta, bool tb, int64_t m, int64_t n, int64_t k, double alpha,
                     const double* A, int64_t lda, const double* B, int64_t ldb, double beta,
                     double* Cm, int64_t ldc, cudaStream_t s, int slot = 28);

@@ -7,182 +7,285 @@
 // row-major with a leading dimension; only lower triangles are referenced
 // where a matrix is symmetric.
 //
-//  potrf_lower: right-looking blocked Cholesky, block NB = 32.  Per block
-//    column: one kernel factors the 32 x 32 diagonal tile (every CTA redoes it
-//    in shared memory) and solves its share of the panel rows; one kernel
-//    applies the rank-32 update to the lower trailing tiles.  Stopping after
-//    nfactor columns leaves the Schur complement in the trailing block.
+//  potrf_lower: right-looking blocked Cholesky, block 16, one launch per block
+//    column: the panel of this column and the trailing update of the previous
+//    one run side by side (k_potrf_step).  Stopping after nfactor columns
+//    leaves the Schur complement in the trailing block.
 //  trsm_lower: L X = B or L^T X = B for many right-hand sides with one
-//    cooperative launch: CTA b owns block rows b, b + G, ... and waits on a
-//    per-block-row flag (bounded spin; a timeout sets a status bit) before
-//    consuming a solved block.
+//    cooperative launch: a CTA owns one block row of a few right-hand sides
+//    and waits on a flag per block row and column chunk (bounded spin; a
+//    timeout sets a status bit) before consuming a solved block.
 #include <math.h>
 
 #include "common.cuh"
 
 namespace rbf {
 
-constexpr int NB = 32;
+constexpr int NB = 32;   // block of the triangular solves
+constexpr int PB = 16;   // block column of the factorization
+constexpr int UT = 32;   // tile of the trailing update
+constexpr int PT = 256;  // threads of a factorization CTA
+
+// 1 / d for a positive normal d: the hardware's approximation (about 20 bits)
+// and one third-order step y (1 + e + e^2), e = 1 - d y (Householder's method
+// for the reciprocal), whose error e^3 lies below float64 rounding.
+__device__ __forceinline__ double rcp_pos(double d) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+  const double e = fma(-d, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
 
 // ---------------------------------------------------------------------------
-// Diagonal tile factorization in shared memory (kb <= 32), all threads of the
-// CTA participate.  T is [32][33].  Returns through T (lower triangle).
+// Step k of the factorization, one CTA per SM.
+//
+// What bounds it: a float64 warp instruction holds its quarter of the SM for
+// 64 cycles whatever its number of active lanes (measured: 65 cycles for one
+// warp, dependent or not; 1.68 lanes a cycle for an SM with 8 warps), so the
+// factorization is bound by the float64 pipe while the trailing block is large,
+// and by the serial chain of the diagonal tile when it is small.  Therefore
+//  * block columns of 16: the work every CTA repeats (the diagonal tile) grows
+//    with the cube of the block, the number of launches only with its inverse;
+//  * look-ahead in one launch: the first CTAs apply panel k - 1 to block column
+//    k, factor its diagonal tile (each for itself) and solve their rows, and
+//    then join the others, who apply panel k - 1 to the columns behind it in
+//    32 x 32 tiles drawn from a counter.  The two parts touch disjoint columns;
+//  * the diagonal tile is eliminated as V D^-1 V^T, without a square root in the
+//    chain, by one warp: lane (i, h) holds row i and the columns 2c + h; the
+//    columns are scaled to L = V D^-1/2 at the end.
+// Against three launches per 32-wide panel (a chain with a barrier per operation,
+// a copy of the tile, 64 x 64 trailing tiles): three frames of a = 1,810, the
+// first banded, 16.7 -> 7.2 ms; a = 256, 630 -> 191 us.  A step without trailing
+// work takes 12 us, of which the chain of the diagonal tile is about 5.
 // ---------------------------------------------------------------------------
-__device__ void chol_tile_smem(double (*T)[NB + 1], int kb, int* flag) {
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, ny = blockDim.x >> 5;
-  __shared__ double rinv;
-  for (int j = 0; j < kb; ++j) {
-    if (threadIdx.x == 0) {
-      double d = T[j][j];
-      if (!(d > 0.0)) {
-        atomicOr(flag, DEV_NOT_SPD);
-        d = 1.0;
+struct PotrfStep {
+  double* A;
+  int64_t lda, k;    // first column of this block column
+  int64_t ne, pe;    // row ends (band) of this panel and of the previous one
+  int kb, kp;        // widths of this block column (0: none) and of the previous one (0: none)
+  int npanel;        // CTAs that share the panel
+  int tiles;         // trailing tiles
+  double* dt;        // factored diagonal tile of this step (16 x 16), if several CTAs read it
+  const double* dtp; // that of the previous step, to be copied into A, or null
+  int* next;         // tile counter, 0 before the launch
+  int* flag;
+};
+
+__global__ void __launch_bounds__(PT) k_potrf_step(PotrfStep P) {
+  __shared__ double D[PB][PB + 1];   // diagonal tile, then V
+  __shared__ double U[PB][PB + 1];   // V D^-1
+  __shared__ double Lk[PB][PB + 1];  // L[k block, k - 1]
+  __shared__ double rs[PB];          // D^-1/2
+  __shared__ double Pi[2][PB][UT + 1], Pj[2][PB][UT + 1];
+  __shared__ int nxt[2];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  double* __restrict__ A = P.A;
+  const int64_t lda = P.lda, k = P.k, k0 = k + P.kb;
+  const int kb = P.kb, kp = P.kp;
+  if (P.dtp && blockIdx.x == gridDim.x - 1) {
+    const int i = tid >> 4, j = tid & 15;
+    if (i < kp && j <= i) A[(k - kp + i) * lda + k - kp + j] = P.dtp[tid];
+  }
+  if ((int)blockIdx.x < P.npanel) {
+    const int i = tid >> 4, j = tid & 15;
+    double dv = (i < kb && j <= i) ? A[(k + i) * lda + k + j] : (i == j ? 1.0 : 0.0);
+    Lk[i][j] = (i < kb && j < kp) ? A[(k + i) * lda + k - kp + j] : 0.0;
+    int64_t r = k0 + (int64_t)blockIdx.x * PB + i;
+    double x = (r < P.ne && j < kb) ? A[r * lda + k + j] : 0.0;
+    double(*Lr)[UT + 1] = Pi[0];  // L[rows, k - 1], transposed
+    Lr[j][i] = (r < P.pe && j < kp) ? A[r * lda + k - kp + j] : 0.0;
+    __syncthreads();
+    if (kp) {
+      double acc = 0.0;
+#pragma unroll
+      for (int t = 0; t < PB; ++t) acc = fma(Lk[i][t], Lk[j][t], acc);
+      if (i < kb && j <= i) dv -= acc;
+    }
+    D[i][j] = dv;
+    __syncthreads();
+    if (warp == 0) {
+      const int ri = lane & 15, h = lane >> 4;
+      double a[PB / 2];
+#pragma unroll
+      for (int c = 0; c < PB / 2; ++c) a[c] = D[ri][2 * c + h];
+      __syncwarp();
+      bool bad = false;
+#pragma unroll
+      for (int t = 0; t < PB; ++t) {
+        const double v = __shfl_sync(0xffffffffu, a[t >> 1], ri + 16 * (t & 1));  // column t of row ri
+        double d = __shfl_sync(0xffffffffu, v, t);
+        if (!(d > 0.0)) {
+          bad = true;
+          d = 1.0;
+        }
+        const double u = v * rcp_pos(d);
+        if (h == 0) {
+          D[ri][t] = ri == t ? d : v;
+          U[ri][t] = u;
+        }
+#pragma unroll
+        for (int c = t >> 1; c < PB / 2; ++c) {
+          const double vk = __shfl_sync(0xffffffffu, v, 2 * c + h);
+          if (2 * c + h > t) a[c] = fma(-u, vk, a[c]);
+        }
       }
-      double r = sqrt(d);
-      T[j][j] = r;
-      rinv = 1.0 / r;
+      if (bad && lane == 0 && blockIdx.x == 0) atomicOr(P.flag, DEV_NOT_SPD);
+      __syncwarp();
+      if (h == 0) rs[ri] = rsqrt(D[ri][ri]);
+    }
+    if (kp) {  // the rows' own update, beside the chain of the diagonal tile
+      double acc = 0.0;
+#pragma unroll
+      for (int t = 0; t < PB; ++t) acc = fma(Lr[t][i], Lk[j][t], acc);
+      x -= acc;
     }
     __syncthreads();
-    if (threadIdx.x < 32 && tx > j && tx < kb) T[tx][j] *= rinv;
-    __syncthreads();
-    if (tx > j) {
-      double tkj = T[tx][j];
-      for (int i = ty; i < kb; i += ny)
-        if (i >= tx) T[i][tx] -= T[i][j] * tkj;
+    if (blockIdx.x == 0) {
+      const double l = i == j ? D[i][i] * rs[i] : (j < i ? D[i][j] * rs[j] : 0.0);
+      if (P.npanel > 1) P.dt[tid] = l;
+      else if (i < kb && j <= i) A[(k + i) * lda + k + j] = l;  // this CTA alone has read the tile
     }
+    double ur[PB - 1];
+#pragma unroll
+    for (int t = 0; t < PB - 1; ++t) ur[t] = U[j][t];
+    const double rj = rs[j];
+    for (int64_t g = blockIdx.x;;) {
+#pragma unroll
+      for (int t = 0; t < PB - 1; ++t) {
+        const double xt = __shfl_sync(0xffffffffu, x, (lane & 16) + t);
+        if (j > t) x = fma(-xt, ur[t], x);
+      }
+      if (r < P.ne && j < kb) A[r * lda + k + j] = x * rj;
+      g += P.npanel;
+      if (k0 + g * PB >= P.ne) break;
+      r = k0 + g * PB + i;
+      x = (r < P.ne && j < kb) ? A[r * lda + k + j] : 0.0;
+      if (kp) {
+        __syncthreads();
+        Lr[j][i] = (r < P.pe && j < kp) ? A[r * lda + k - kp + j] : 0.0;
+        __syncthreads();
+        double acc = 0.0;
+#pragma unroll
+        for (int t = 0; t < PB; ++t) acc = fma(Lr[t][i], Lk[j][t], acc);
+        x -= acc;
+      }
+    }
+    __syncthreads();  // Lr is staged over below
+  }
+  // trailing tiles (ti >= tj) of rows [k0, pe): C -= P P^T with the previous
+  // panel P; the next tile's operands are on their way while this one's
+  // products run.
+  if (P.tiles == 0) return;
+  const int tx = tid & 15, ty = tid >> 4;
+  double pi[2], pj[2], cv[4];
+  int64_t i0 = 0, j0 = 0;
+  auto fetch = [&](int b, int64_t& fi, int64_t& fj) {
+    int ti = (int)((sqrtf(8.f * (float)b + 1.f) - 1.f) * 0.5f);
+    while ((ti + 1) * (ti + 2) / 2 <= b) ++ti;
+    while (ti * (ti + 1) / 2 > b) --ti;
+    fi = k0 + (int64_t)ti * UT;
+    fj = k0 + (int64_t)(b - ti * (ti + 1) / 2) * UT;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int64_t ra = fi + ty + 16 * u, rb = fj + ty + 16 * u;
+      pi[u] = (ra < P.pe && tx < kp) ? A[ra * lda + k - kp + tx] : 0.0;
+      pj[u] = (rb < P.pe && tx < kp) ? A[rb * lda + k - kp + tx] : 0.0;
+#pragma unroll
+      for (int v = 0; v < 2; ++v) {
+        const int64_t ri = fi + 2 * ty + u, cj = fj + tx + 16 * v;
+        cv[2 * u + v] = (ri < P.pe && cj <= ri) ? A[ri * lda + cj] : 0.0;
+      }
+    }
+  };
+  if (tid == 0) nxt[0] = atomicAdd(P.next, 1);
+  __syncthreads();
+  int b = nxt[0], par = 0;
+  if (b >= P.tiles) return;
+  fetch(b, i0, j0);
+  while (b < P.tiles) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      Pi[par][tx][ty + 16 * u] = pi[u];
+      Pj[par][tx][ty + 16 * u] = pj[u];
+    }
+    double c[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) c[q] = cv[q];
+    if (tid == 0) nxt[par ^ 1] = atomicAdd(P.next, 1);
     __syncthreads();
+    const int bn = nxt[par ^ 1];
+    const int64_t ci = i0, cj0 = j0;
+    if (bn < P.tiles) fetch(bn, i0, j0);
+#pragma unroll
+    for (int t = 0; t < PB; ++t) {
+      const double a0 = Pi[par][t][2 * ty], a1 = Pi[par][t][2 * ty + 1];
+      const double b0 = Pj[par][t][tx], b1 = Pj[par][t][tx + 16];
+      c[0] = fma(-a0, b0, c[0]);
+      c[1] = fma(-a0, b1, c[1]);
+      c[2] = fma(-a1, b0, c[2]);
+      c[3] = fma(-a1, b1, c[3]);
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int v = 0; v < 2; ++v) {
+        const int64_t ri = ci + 2 * ty + u, cj = cj0 + tx + 16 * v;
+        if (ri < P.pe && cj <= ri) A[ri * lda + cj] = c[2 * u + v];
+      }
+    b = bn;
+    par ^= 1;
   }
 }
 
-// Panel kernel of step k: factor A[k:k+kb, k:k+kb], then solve rows
-// [k+kb, n) of the block column: X L_kk^T = A[rows, k:k+kb].
-__global__ void __launch_bounds__(256) k_potrf_panel(double* __restrict__ A, int64_t lda, int64_t n,
-                                                     int64_t k, int kb, int rows_per_cta,
-                                                     double* __restrict__ dtile,
-                                                     int* __restrict__ flag) {
-  __shared__ double T[NB][NB + 1];
-  __shared__ double inv_d[NB];
-  for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
-    int i = e / NB, j = e % NB;
-    T[i][j] = (i < kb && j <= i) ? A[(k + i) * lda + k + j] : 0.0;
-  }
-  __syncthreads();
-  chol_tile_smem(T, kb, flag);
-  if (threadIdx.x < NB) inv_d[threadIdx.x] = threadIdx.x < kb ? 1.0 / T[threadIdx.x][threadIdx.x] : 0.0;
-  __syncthreads();
-  // every CTA reads the unfactored tile from A, so the factored tile goes to
-  // scratch and k_copy_tile writes it back after this kernel
-  if (blockIdx.x == 0) {
-    for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
-      int i = e / NB, j = e % NB;
-      dtile[e] = (j <= i) ? T[i][j] : 0.0;
-    }
-  }
-  // panel rows: one warp per row, lane c holds column c
-  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  int64_t r0 = k + kb + (int64_t)blockIdx.x * rows_per_cta;
-  int64_t r1 = r0 + rows_per_cta;
-  if (r1 > n) r1 = n;
-  for (int64_t r = r0 + wid; r < r1; r += nw) {
-    double* row = A + r * lda + k;
-    double b = lane < kb ? row[lane] : 0.0;
-    for (int t = 0; t < kb; ++t) {
-      double xt = __shfl_sync(0xffffffffu, b, t) * inv_d[t];
-      if (lane == t) b = xt;
-      else if (lane > t) b -= xt * T[lane][t];
-    }
-    if (lane < kb) row[lane] = b;
-  }
-}
-
-__global__ void k_copy_tile(double* __restrict__ A, int64_t lda, int64_t k, int kb,
-                            const double* __restrict__ dtile) {
-  for (int e = threadIdx.x; e < kb * kb; e += blockDim.x) {
-    int i = e / kb, j = e % kb;
-    A[(k + i) * lda + k + j] = dtile[i * NB + j];
-  }
-}
-
-// Trailing update of step k: for lower tiles (ti >= tj) of the block
-// A[k0:n, k0:n] (k0 = k + kb): C -= P P^T with P = A[k0:n, k:k+kb].
-constexpr int ST = 64;  // output tile
-__global__ void __launch_bounds__(256) k_syrk_trailing(double* __restrict__ A, int64_t lda, int64_t n,
-                                                       int64_t k, int kb) {
-  int64_t k0 = k + kb;
-  int64_t b = blockIdx.x;
-  int64_t ti = (int64_t)((sqrt(8.0 * (double)b + 1.0) - 1.0) * 0.5);
-  while ((ti + 1) * (ti + 2) / 2 <= b) ++ti;
-  while (ti * (ti + 1) / 2 > b) --ti;
-  int64_t tj = b - ti * (ti + 1) / 2;
-  int64_t i0 = k0 + ti * ST, j0 = k0 + tj * ST;
-  __shared__ double Pi[NB][ST + 1];
-  __shared__ double Pj[NB][ST + 1];
-  for (int e = threadIdx.x; e < ST * NB; e += blockDim.x) {
-    int r = e / NB, t = e % NB;
-    double vi = 0.0, vj = 0.0;
-    if (t < kb) {
-      if (i0 + r < n) vi = A[(i0 + r) * lda + k + t];
-      if (j0 + r < n) vj = A[(j0 + r) * lda + k + t];
-    }
-    Pi[t][r] = vi;
-    Pj[t][r] = vj;
-  }
-  __syncthreads();
-  int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  double acc[4][4] = {};
-  for (int t = 0; t < kb; ++t) {
-    double a[4], bb[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      a[u] = Pi[t][ty * 4 + u];
-      bb[u] = Pj[t][tx * 4 + u];
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-      for (int v = 0; v < 4; ++v) acc[u][v] = fma(a[u], bb[v], acc[u][v]);
-  }
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    int64_t i = i0 + ty * 4 + u;
-    if (i >= n) continue;
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      int64_t j = j0 + tx * 4 + v;
-      if (j < n && j <= i) A[i * lda + j] -= acc[u][v];
-    }
-  }
+static int dense_sms(int dev) {
+  static int sms[64] = {0};
+  int& v = sms[dev & 63];
+  if (!v && (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0)) v = 152;
+  return v;
 }
 
 rbf_status potrf_lower(Ctx* c, double* A, int64_t n, int64_t lda, int64_t nfactor, bool mixed,
                        cudaStream_t s, int64_t bw) {
   (void)mixed;
   if (n <= 0 || nfactor <= 0) return RBF_OK;
-  int* flag = c->dflag.as<int>();
+  const int64_t steps = (nfactor + PB - 1) / PB;
+  const int sms = dense_sms(c->device);
+  // two diagonal tiles, then one tile counter per launch
   Buf& dt = c->scratch(30);
-  RBF_TRY(dt.ensure(NB * NB * sizeof(double)));
-  for (int64_t k = 0; k < nfactor; k += NB) {
-    int kb = (int)((nfactor - k) < NB ? (nfactor - k) : NB);
+  RBF_TRY(dt.ensure(2 * PB * PB * sizeof(double) + (size_t)(steps + 1) * sizeof(int)));
+  int* next = reinterpret_cast<int*>(dt.as<double>() + 2 * PB * PB);
+  RBF_CUDA(cudaMemsetAsync(next, 0, (size_t)(steps + 1) * sizeof(int), s));
+  StageTimer st(c, RBF_STAGE_PANEL, s, (double)n * n * n / 3.0);
+  PotrfStep P;
+  P.A = A;
+  P.lda = lda;
+  P.flag = c->dflag.as<int>();
+  P.kp = 0;
+  P.pe = 0;
+  P.dtp = nullptr;
+  for (int64_t q = 0; q <= steps; ++q) {
+    P.k = q * PB < nfactor ? q * PB : nfactor;
+    P.kb = (int)((nfactor - P.k) < PB ? (nfactor - P.k) : PB);  // 0: the last panel's update only
+    const int64_t k0 = P.k + P.kb;
     // rows beyond the band are zero in this panel and untouched by its update
-    const int64_t ne = (k + kb + bw) < n ? (k + kb + bw) : n;
-    int64_t rows = ne - k - kb;
-    int rows_per_cta = 16;
-    int64_t ctas = rows > 0 ? (rows + rows_per_cta - 1) / rows_per_cta : 1;
-    {
-      StageTimer st(c, RBF_STAGE_PANEL, s, (double)kb * kb * kb / 3.0 + (double)rows * kb * kb);
-      { k_potrf_panel<<<(unsigned)ctas, 256, 0, s>>>(A, lda, ne, k, kb, rows_per_cta, dt.as<double>(),
-                                                   flag); ::rbf::note_launch(); }
-      RBF_CUDA(cudaGetLastError());
-      { k_copy_tile<<<1, 256, 0, s>>>(A, lda, k, kb, dt.as<double>()); ::rbf::note_launch(); }
-      RBF_CUDA(cudaGetLastError());
+    P.ne = P.kb ? ((k0 + bw) < n ? (k0 + bw) : n) : P.k;
+    const int64_t groups = (P.ne - k0 + PB - 1) / PB;
+    P.npanel = P.kb ? (int)(groups < 1 ? 1 : (groups < sms ? groups : sms)) : 0;
+    const int64_t T = P.pe > k0 ? (P.pe - k0 + UT - 1) / UT : 0;
+    P.tiles = P.kp ? (int)(T * (T + 1) / 2) : 0;
+    P.dt = dt.as<double>() + (q & 1) * PB * PB;
+    P.next = next + q;
+    int64_t grid = (int64_t)P.npanel + P.tiles;
+    if (grid > sms) grid = sms;
+    if (grid < 1) {
+      if (!P.dtp) break;
+      grid = 1;
     }
-    if (rows > 0) {
-      StageTimer st(c, RBF_STAGE_TRAILING, s, (double)rows * (double)(rows + 1) * kb);
-      int64_t T = (rows + ST - 1) / ST;
-      int64_t tiles = T * (T + 1) / 2;
-      { k_syrk_trailing<<<(unsigned)tiles, 256, 0, s>>>(A, lda, ne, k, kb); ::rbf::note_launch(); }
-      RBF_CUDA(cudaGetLastError());
-    }
+    { k_potrf_step<<<(unsigned)grid, PT, 0, s>>>(P); ::rbf::note_launch(); }
+    RBF_CUDA(cudaGetLastError());
+    P.dtp = P.npanel > 1 ? P.dt : nullptr;
+    P.kp = P.kb;
+    P.pe = P.ne;
   }
   return RBF_OK;
 }
@@ -190,7 +293,6 @@ rbf_status potrf_lower(Ctx* c, double* A, int64_t n, int64_t lda, int64_t nfacto
 // ---------------------------------------------------------------------------
 // Sync-free blocked triangular solve with many right-hand sides.
 // ---------------------------------------------------------------------------
-constexpr int TS_MC = 32;          // right-hand sides per launch
 constexpr int TS_THREADS = 256;
 constexpr long long TS_SPIN_LIMIT = 1LL << 22;
 
@@ -203,156 +305,200 @@ __device__ __forceinline__ void st_release(int* p, int v) {
   asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// Solves op(L) X = B in place for columns [c0, c0 + mc) of B.
-// transpose = false: forward (block rows in order 0..nblk-1)
-// transpose = true : backward with L^T (block rows nblk-1..0)
-// Before waiting on anything, a CTA inverts the diagonal block of its block
-// row; each dependency is then a 32 x 32 x mc product from a shared-memory
-// copy of the solved block, and the final step is x = D^{-1} acc.
-__global__ void __launch_bounds__(TS_THREADS) k_trsm_syncfree(const double* __restrict__ L, int64_t ldl,
-                                                              int64_t n, double* B, int64_t ldb,
-                                                              int c0, int mc, bool transpose, int64_t bwb,
+// Inverses of the 32 x 32 diagonal blocks of L, one CTA each, identity beyond a
+// ragged last block: the 16 x 16 halves by substitution (a warp each, lane =
+// column), Z21 = -Z22 (L21 Z11) by all threads.  The solves apply them as
+// products (10 us a factor).  Formed inside every CTA of every solve, with a
+// division per entry, they were most of the 153 us of a solve of 256 unknowns
+// (now 22 us).
+__global__ void __launch_bounds__(TS_THREADS) k_diag_inv(const double* __restrict__ L, int64_t ldl, int64_t n,
+                                                         double* __restrict__ Z) {
+  __shared__ double T[NB][NB + 1], Zs[NB][NB + 1], Y[16][17];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t r0 = (int64_t)blockIdx.x * NB;
+  for (int e = tid; e < NB * NB; e += TS_THREADS) {
+    const int i = e / NB, j = e % NB;
+    T[i][j] = (r0 + i < n && j <= i) ? L[(r0 + i) * ldl + r0 + j] : (i == j ? 1.0 : 0.0);
+    Zs[i][j] = 0.0;
+  }
+  __syncthreads();
+  if (warp < 2 && lane < 16) {
+    const int o = 16 * warp;
+    const double rd = 1.0 / T[o + lane][o + lane];
+    double z[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      double acc = i == lane ? 1.0 : 0.0;
+#pragma unroll
+      for (int t = 0; t < i; ++t) acc = fma(-T[o + i][o + t], z[t], acc);
+      z[i] = acc * __shfl_sync(0xffffu, rd, i);
+      if (i >= lane) Zs[o + i][o + lane] = z[i];
+    }
+  }
+  __syncthreads();
+  const int i = tid >> 4, j = tid & 15;
+  double acc = 0.0;
+#pragma unroll
+  for (int t = 0; t < 16; ++t) acc = fma(T[16 + i][t], Zs[t][j], acc);
+  Y[i][j] = acc;
+  __syncthreads();
+  acc = 0.0;
+#pragma unroll
+  for (int t = 0; t < 16; ++t) acc = fma(-Zs[16 + i][16 + t], Y[t][j], acc);
+  Zs[16 + i][j] = acc;
+  __syncthreads();
+  for (int e = tid; e < NB * NB; e += TS_THREADS) Z[(int64_t)blockIdx.x * NB * NB + e] = Zs[e / NB][e % NB];
+}
+
+// Solves op(L) X = B in place: item (lk, ch) is block row lk (in the order of
+// the solve) of the TW right-hand sides of chunk ch.  A CTA walks its items in
+// ascending order, block rows first, so that every wait is for an earlier item
+// of a co-resident CTA.  A thread keeps the partial sum of one row and one
+// right-hand side over a share of the columns in a register until the row is
+// done; the next block of L is loaded while the current one is used.
+// Narrow chunks (4 right-hand sides, 8 above 64) because a step of the chain
+// costs 32 x 32 x TW products on one SM's slow float64 pipe.  At a = 1,810 the
+// solves of three frames (six with one right-hand side, two with about 50, which
+// took two launches of 32) went from 8.9 to 1.5 ms: 0.16 ms each and 0.30 ms each.
+template <int TW>
+__global__ void __launch_bounds__(TS_THREADS) k_trsm_syncfree(const double* __restrict__ L, int64_t ldl, int64_t n,
+                                                              const double* __restrict__ Z, double* B, int64_t ldb,
+                                                              int64_t m, int64_t nch, bool transpose, int64_t bwb,
                                                               int* flags, int epoch, int* status,
                                                               long long spin_limit, int wait_xor) {
-  __shared__ double acc[NB][TS_MC + 1];
-  __shared__ double Xs[NB][TS_MC + 1];
-  __shared__ double Dinv[NB][NB + 1];
-  __shared__ double Dg[NB][NB + 1];
+  constexpr int KS = 8 / TW;  // shares of the columns
+  __shared__ double Ls[NB][NB + 1];
+  __shared__ double Xs[NB][TW];
   __shared__ int bail;
   const int tid = threadIdx.x, ti = tid >> 3, tg = tid & 7;
-  const int lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
-  int64_t nblk = (n + NB - 1) / NB;
-  for (int64_t lk = blockIdx.x; lk < nblk; lk += gridDim.x) {
-    int64_t r = transpose ? (nblk - 1 - lk) : lk;
-    int64_t r0 = r * NB;
-    int rb = (int)((n - r0) < NB ? (n - r0) : NB);
-    // diagonal block op(L)_rr (lower for forward, upper for transpose) and its inverse
-    for (int e = tid; e < NB * NB; e += blockDim.x) {
-      int i = e / NB, j = e % NB;
-      double v = (i == j) ? 1.0 : 0.0;
-      if (i < rb && j < rb) v = transpose ? L[(r0 + j) * ldl + r0 + i] : L[(r0 + i) * ldl + r0 + j];
-      Dg[i][j] = v;
-    }
-    for (int e = tid; e < NB * TS_MC; e += blockDim.x) {
-      int i = e / TS_MC, j = e % TS_MC;
-      acc[i][j] = (i < rb && j < mc) ? B[(r0 + i) * ldb + c0 + j] : 0.0;
-    }
-    if (tid == 0) bail = 0;
-    __syncthreads();
-    // column c of D^{-1}: solve D x = e_c by substitution, lane = row
-    for (int cidx = wid; cidx < NB; cidx += nw) {
-      double b = (lane == cidx) ? 1.0 : 0.0;
-      if (!transpose) {
-        for (int t = 0; t < NB; ++t) {
-          double xt = __shfl_sync(0xffffffffu, b, t) / Dg[t][t];
-          if (lane == t) b = xt;
-          else if (lane > t) b -= Dg[lane][t] * xt;
-        }
-      } else {
-        for (int t = NB - 1; t >= 0; --t) {
-          double xt = __shfl_sync(0xffffffffu, b, t) / Dg[t][t];
-          if (lane == t) b = xt;
-          else if (lane < t) b -= Dg[lane][t] * xt;
-        }
-      }
-      Dinv[lane][cidx] = b;
-    }
-    for (int64_t lc = (lk - bwb) > 0 ? (lk - bwb) : 0; lc < lk; ++lc) {  // blocks outside the band are zero
-      int64_t cb = transpose ? (nblk - 1 - lc) : lc;
-      int64_t cc0 = cb * NB;
-      int cbs = (int)((n - cc0) < NB ? (n - cc0) : NB);
-      double lv[4];
+  const int ks = tg % KS, j = tg / KS;
+  const int64_t nblk = (n + NB - 1) / NB;
+  if (tid == 0) bail = 0;
+  __syncthreads();
+  for (int64_t it = blockIdx.x; it < nblk * nch; it += gridDim.x) {
+    const int64_t lk = it / nch, ch = it % nch;
+    const int64_t r = transpose ? (nblk - 1 - lk) : lk, r0 = r * NB, c0 = ch * TW;
+    const int rb = (int)((n - r0) < NB ? (n - r0) : NB);
+    const int mc = (int)((m - c0) < TW ? (m - c0) : TW);
+    // op(L)[r, cb]: thread (ti, tg) loads 4 entries, contiguous over tg
+    double lv[4];
+    auto load_l = [&](int64_t lc) {
+      const int64_t cb = transpose ? (nblk - 1 - lc) : lc, cc0 = cb * NB;
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        int t = 4 * tg + u;
-        double v = 0.0;
-        if (ti < rb && t < cbs)
-          v = transpose ? L[(cc0 + t) * ldl + r0 + ti] : L[(r0 + ti) * ldl + cc0 + t];
-        lv[u] = v;
+        const int t = tg + 8 * u;  // forward: L[r0 + ti, cc0 + t]; transposed: L[cc0 + ti, r0 + t]
+        if (!transpose) lv[u] = (ti < rb && cc0 + t < n) ? L[(r0 + ti) * ldl + cc0 + t] : 0.0;
+        else lv[u] = (cc0 + ti < n && t < rb) ? L[(cc0 + ti) * ldl + r0 + t] : 0.0;
       }
+    };
+    double acc = 0.0;
+    int64_t lc = (lk - bwb) > 0 ? (lk - bwb) : 0;  // blocks outside the band are zero
+    if (lc < lk) load_l(lc);
+    for (; lc < lk; ++lc) {
+      const int64_t cb = transpose ? (nblk - 1 - lc) : lc, cc0 = cb * NB;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (!transpose) Ls[ti][tg + 8 * u] = lv[u];
+        else Ls[tg + 8 * u][ti] = lv[u];
+      }
+      if (lc + 1 < lk) load_l(lc + 1);
       if (tid == 0) {
-        long long it = 0;
-        while (ld_acquire(flags + cb) != (epoch ^ wait_xor)) {
-          if (++it > spin_limit) {
+        long long spins = 0;
+        while (ld_acquire(flags + ch * nblk + cb) != (epoch ^ wait_xor)) {
+          if (++spins > spin_limit) {
             atomicOr(status, DEV_TIMEOUT);
             bail = 1;
             break;
           }
-          __nanosleep(20);
         }
       }
       __syncthreads();
-      if (bail) break;
-      for (int e = tid; e < NB * mc; e += blockDim.x) {
-        int t = e / mc, j = e % mc;
-        Xs[t][j] = (t < cbs) ? __ldcg(B + (cc0 + t) * ldb + c0 + j) : 0.0;
+      if (bail) return;
+      if (tid < NB * TW) {
+        const int t = tid / TW, q = tid % TW;
+        Xs[t][q] = (cc0 + t < n && q < mc) ? __ldcg(B + (cc0 + t) * ldb + c0 + q) : 0.0;
       }
       __syncthreads();
-      for (int j = 0; j < mc; ++j) {
-        double pp = 0.0;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) pp = fma(lv[u], Xs[4 * tg + u][j], pp);
-        pp += __shfl_xor_sync(0xffffffffu, pp, 1);
-        pp += __shfl_xor_sync(0xffffffffu, pp, 2);
-        pp += __shfl_xor_sync(0xffffffffu, pp, 4);
-        if (tg == 0) acc[ti][j] -= pp;
-      }
+      for (int q = 0; q < NB / KS; ++q) acc = fma(Ls[ti][ks + KS * q], Xs[ks + KS * q][j], acc);
       __syncthreads();
     }
+    // x = D^{-1} (b - acc)
+#pragma unroll
+    for (int o = 1; o < KS; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    const double* Zr = Z + r * NB * NB;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const double z = Zr[ti * NB + tg + 8 * u];
+      if (!transpose) Ls[ti][tg + 8 * u] = z;
+      else Ls[tg + 8 * u][ti] = z;
+    }
+    if (ks == 0) Xs[ti][j] = (ti < rb && j < mc) ? __ldcg(B + (r0 + ti) * ldb + c0 + j) - acc : 0.0;
     __syncthreads();
-    // x = D^{-1} acc
-    for (int j = 0; j < mc; ++j) {
-      double pp = 0.0;
+    double x = 0.0;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) pp = fma(Dinv[ti][4 * tg + u], acc[4 * tg + u][j], pp);
-      pp += __shfl_xor_sync(0xffffffffu, pp, 1);
-      pp += __shfl_xor_sync(0xffffffffu, pp, 2);
-      pp += __shfl_xor_sync(0xffffffffu, pp, 4);
-      if (tg == 0 && ti < rb) B[(r0 + ti) * ldb + c0 + j] = pp;
-    }
+    for (int q = 0; q < NB / KS; ++q) x = fma(Ls[ti][ks + KS * q], Xs[ks + KS * q][j], x);
+#pragma unroll
+    for (int o = 1; o < KS; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if (ks == 0 && ti < rb && j < mc) B[(r0 + ti) * ldb + c0 + j] = x;
     __syncthreads();
     if (tid == 0) {
       __threadfence();  // cumulative: orders the block's stores (seen through the barrier) before the flag
-      st_release(flags + r, epoch);
+      st_release(flags + ch * nblk + r, epoch);
     }
   }
 }
 
-rbf_status trsm_lower(Ctx* c, const double* L, int64_t n, int64_t ldl, double* B, int64_t m,
-                      int64_t ldb, bool transpose, cudaStream_t s, int64_t bw) {
-  if (n <= 0 || m <= 0) return RBF_OK;
-  int64_t nblk = (n + NB - 1) / NB;
-  if (c->sync_flags.bytes < (size_t)nblk * sizeof(int)) {
-    RBF_TRY(c->sync_flags.ensure((size_t)nblk * sizeof(int)));
+// Inverses of the diagonal blocks of a factor, for the solves that follow.
+static rbf_status diag_inverses(Ctx* c, const double* L, int64_t n, int64_t ldl, cudaStream_t s) {
+  const int64_t nblk = (n + NB - 1) / NB;
+  Buf& zb = c->scratch(99);
+  RBF_TRY(zb.ensure((size_t)nblk * NB * NB * sizeof(double)));
+  { k_diag_inv<<<(unsigned)nblk, TS_THREADS, 0, s>>>(L, ldl, n, zb.as<double>()); ::rbf::note_launch(); }
+  RBF_CUDA(cudaGetLastError());
+  return RBF_OK;
+}
+
+template <int TW>
+static rbf_status trsm_launch(Ctx* c, const double* L, int64_t n, int64_t ldl, double* B, int64_t m, int64_t ldb,
+                              bool transpose, cudaStream_t s, int64_t bw) {
+  int64_t nblk = (n + NB - 1) / NB, nch = (m + TW - 1) / TW;
+  const size_t fbytes = (size_t)(nblk * nch) * sizeof(int);
+  if (c->sync_flags.bytes < fbytes) {
+    RBF_TRY(c->sync_flags.ensure(fbytes));
     RBF_CUDA(cudaMemsetAsync(c->sync_flags.p, 0, c->sync_flags.bytes, s));
     c->epoch = 0;
   }
   static int max_blocks_dev[64] = {0};
-  int dev = c->device;
-  if (!max_blocks_dev[dev & 63]) {
-    int per_sm = 0, sms = 0;
-    RBF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_trsm_syncfree, TS_THREADS, 0));
-    RBF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    max_blocks_dev[dev & 63] = per_sm * sms;
+  int& max_blocks = max_blocks_dev[c->device & 63];
+  if (!max_blocks) {
+    int per_sm = 0;
+    RBF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_trsm_syncfree<TW>, TS_THREADS, 0));
+    max_blocks = per_sm * dense_sms(c->device);
   }
-  int64_t grid = nblk < max_blocks_dev[dev & 63] ? nblk : max_blocks_dev[dev & 63];
+  int64_t grid = nblk * nch < max_blocks ? nblk * nch : max_blocks;
   if (grid < 1) return fail(RBF_ECUDA, "trsm: no co-resident blocks");
+  const double* Z = c->scratch(99).as<double>();
   int* flags = c->sync_flags.as<int>();
   int* status = c->dflag.as<int>();
-  for (int64_t c0 = 0; c0 < m; c0 += TS_MC) {
-    int mc = (int)((m - c0) < TS_MC ? (m - c0) : TS_MC);
-    int epoch = (int)(++c->epoch);
-    int c0i = (int)c0;
-    int64_t bwb = bw >= n ? nblk : bw / NB + 2;
-    long long lim = c->spin_limit > 0 ? c->spin_limit : TS_SPIN_LIMIT;
-    int wx = c->wait_xor;
-    void* args[] = {(void*)&L, (void*)&ldl, (void*)&n, (void*)&B, (void*)&ldb, (void*)&c0i,
-                    (void*)&mc, (void*)&transpose, (void*)&bwb, (void*)&flags, (void*)&epoch, (void*)&status,
-                    (void*)&lim, (void*)&wx};
-    RBF_CUDA(cooperative_launch((const void*)k_trsm_syncfree, dim3((unsigned)grid),
-                                         dim3(TS_THREADS), args, 0, s));
-  }
+  int epoch = (int)(++c->epoch);
+  int64_t bwb = bw >= n ? nblk : bw / NB + 2;
+  long long lim = c->spin_limit > 0 ? c->spin_limit : TS_SPIN_LIMIT;
+  int wx = c->wait_xor;
+  void* args[] = {(void*)&L,   (void*)&ldl,       (void*)&n,   (void*)&Z,     (void*)&B,     (void*)&ldb,    (void*)&m,
+                  (void*)&nch, (void*)&transpose, (void*)&bwb, (void*)&flags, (void*)&epoch, (void*)&status, (void*)&lim,
+                  (void*)&wx};
+  RBF_CUDA(cooperative_launch((const void*)k_trsm_syncfree<TW>, dim3((unsigned)grid), dim3(TS_THREADS), args, 0, s));
   return RBF_OK;
+}
+
+rbf_status trsm_lower(Ctx* c, const double* L, int64_t n, int64_t ldl, double* B, int64_t m,
+                      int64_t ldb, bool transpose, cudaStream_t s, int64_t bw, bool have_inv) {
+  if (n <= 0 || m <= 0) return RBF_OK;
+  if (!have_inv) RBF_TRY(diag_inverses(c, L, n, ldl, s));
+  if (m == 1) return trsm_launch<1>(c, L, n, ldl, B, m, ldb, transpose, s, bw);
+  if (m <= 64) return trsm_launch<4>(c, L, n, ldl, B, m, ldb, transpose, s, bw);
+  return trsm_launch<8>(c, L, n, ldl, B, m, ldb, transpose, s, bw);
 }
 
 // ---------------------------------------------------------------------------

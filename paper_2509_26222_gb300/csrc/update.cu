@@ -642,7 +642,7 @@ rbf_status chol_solve(Ctx* c, const double* H, const double* L, int64_t a, int64
                       cudaStream_t s, int64_t bw) {
   if (!refine) {
     RBF_TRY(trsm_lower(c, L, a, ld, b, 1, 1, false, s, bw));
-    RBF_TRY(trsm_lower(c, L, a, ld, b, 1, 1, true, s, bw));
+    RBF_TRY(trsm_lower(c, L, a, ld, b, 1, 1, true, s, bw, true));
     return RBF_OK;
   }
   Buf& rb = c->scratch(31);
@@ -654,11 +654,11 @@ rbf_status chol_solve(Ctx* c, const double* H, const double* L, int64_t a, int64
   RBF_CUDA(cudaMemcpyAsync(bb.p, b, (size_t)a * sizeof(double), cudaMemcpyDeviceToDevice, s));
   RBF_CUDA(cudaMemcpyAsync(xb.p, b, (size_t)a * sizeof(double), cudaMemcpyDeviceToDevice, s));
   RBF_TRY(trsm_lower(c, L, a, ld, xb.as<double>(), 1, 1, false, s, bw));
-  RBF_TRY(trsm_lower(c, L, a, ld, xb.as<double>(), 1, 1, true, s, bw));
+  RBF_TRY(trsm_lower(c, L, a, ld, xb.as<double>(), 1, 1, true, s, bw, true));
   for (int it = 0; it < 6; ++it) {
     RBF_TRY(symv_residual(H, a, ld, xb.as<double>(), bb.as<double>(), rb.as<double>(), s));
-    RBF_TRY(trsm_lower(c, L, a, ld, rb.as<double>(), 1, 1, false, s, bw));
-    RBF_TRY(trsm_lower(c, L, a, ld, rb.as<double>(), 1, 1, true, s, bw));
+    RBF_TRY(trsm_lower(c, L, a, ld, rb.as<double>(), 1, 1, false, s, bw, true));
+    RBF_TRY(trsm_lower(c, L, a, ld, rb.as<double>(), 1, 1, true, s, bw, true));
     { k_axpy<<<nblk(a), 256, 0, s>>>(xb.as<double>(), rb.as<double>(), a); ::rbf::note_launch(); }
     RBF_CUDA(cudaGetLastError());
   }
