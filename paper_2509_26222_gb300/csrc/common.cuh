@@ -313,7 +313,7 @@ rbf_status mixed_cov(Ctx* c, const double* H, int64_t ldh, const SpH* Hs, const 
                      const float* Zd, const float* Zi, int64_t n, double* B, int64_t k, const int32_t* pos,
                      int sweeps, double* P, cudaStream_t s, int64_t bw = BW_DENSE);
 // compressed rows of the information matrix (sparse.cu)
-rbf_status build_csr(Ctx* c, const double* H, int64_t ld, int64_t n, SpH& out, cudaStream_t s);
+rbf_status build_csr(Ctx* c, const double* H, int64_t ld, int64_t n, int64_t band, SpH& out, cudaStream_t s);
 rbf_status csr_bandwidth(Ctx* c, int64_t n, int64_t* bw, cudaStream_t s);
 rbf_status dense_bandwidth(Ctx* c, const double* H, int64_t ld, int64_t n, int64_t* bw, cudaStream_t s);
 rbf_status csr_residual(const SpH& A, const double* X, const double* B, int64_t m, double* R, cudaStream_t s);
@@ -345,7 +345,7 @@ void bq_destroy(void* state);
 // forget the cached device address of rbf_soft_cost_noalloc's scratch on `dev`
 void noalloc_forget(int dev);
 rbf_status symv_residual(const double* H, int64_t n, int64_t ld, const double* x,
-                         const double* b, double* r, cudaStream_t s);
+                         const double* b, double* r, cudaStream_t s, int64_t bw = BW_DENSE);
 
 }  // namespace rbf
 

@@ -663,8 +663,8 @@ rbf_status gemm_f64(Ctx* c, bool ta, bool tb, int64_t m, int64_t n, int64_t k, d
   return RBF_OK;
 }
 
-// r = b - H x for a symmetric H stored in full (one warp per row).
-__global__ void __launch_bounds__(256) k_symv_residual(const double* __restrict__ H, int64_t n, int64_t ld,
+// r = b - H x for a symmetric H stored in full (one warp per row, its band only).
+__global__ void __launch_bounds__(256) k_symv_residual(const double* __restrict__ H, int64_t n, int64_t ld, int64_t bw,
                                                        const double* __restrict__ x,
                                                        const double* __restrict__ b,
                                                        double* __restrict__ r) {
@@ -672,16 +672,17 @@ __global__ void __launch_bounds__(256) k_symv_residual(const double* __restrict_
   int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (row >= n) return;
   double acc = 0.0;
-  for (int64_t j = lane; j < n; j += 32) acc = fma(H[row * ld + j], x[j], acc);
+  const int64_t j1 = row + bw < n ? row + bw + 1 : n;
+  for (int64_t j = (row > bw ? row - bw : 0) + lane; j < j1; j += 32) acc = fma(H[row * ld + j], x[j], acc);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
   if (lane == 0) r[row] = b[row] - acc;
 }
 
 rbf_status symv_residual(const double* H, int64_t n, int64_t ld, const double* x, const double* b,
-                         double* r, cudaStream_t s) {
+                         double* r, cudaStream_t s, int64_t bw) {
   if (n <= 0) return RBF_OK;
-  { k_symv_residual<<<(unsigned)((n * 32 + 255) / 256), 256, 0, s>>>(H, n, ld, x, b, r); ::rbf::note_launch(); }
+  { k_symv_residual<<<(unsigned)((n * 32 + 255) / 256), 256, 0, s>>>(H, n, ld, bw, x, b, r); ::rbf::note_launch(); }
   RBF_CUDA(cudaGetLastError());
   return RBF_OK;
 }

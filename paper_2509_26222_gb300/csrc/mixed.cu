@@ -34,6 +34,17 @@ __global__ void k_mx_to_f32(const double* __restrict__ H, int64_t ldh, int64_t n
   W[i * ldw + j] = (float)H[i * ldh + j];
 }
 
+// The same for the part of a banded H that the factorization and the solves
+// read: columns [i - bw - 191, i + 127] (whole 64 x 64 tiles up to two block
+// columns past the band, and the diagonal tile of a 128-wide update).
+// a = 8,189, bw = 390: 235 -> 30 us.
+__global__ void k_mx_to_f32_band(const double* __restrict__ H, int64_t ldh, int64_t n, int64_t below,
+                                 float* __restrict__ W, int64_t ldw) {
+  const int64_t i = blockIdx.y, j = i - below + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (j < 0 || j >= n || j > i + 127) return;
+  W[i * ldw + j] = (float)H[i * ldh + j];
+}
+
 // ---------------------------------------------------------------------------
 // One block column of the factorization in one launch.  Every CTA factors the
 // 64 x 64 diagonal tile W_kk itself (L_kk, and Z_kk = L_kk^{-1}), then
@@ -552,8 +563,18 @@ static rbf_status potrf_df(Ctx* c, int64_t n, float* W, int64_t ldw, float* Zd, 
 
 static rbf_status potrf_chain(Ctx* c, int64_t n, float* W, int64_t ldw, float* Zd, cudaStream_t s, int64_t bw);
 
-static rbf_status to_f32(const double* H, int64_t ldh, int64_t n, float* W, int64_t ldw, cudaStream_t s) {
+// band_only: nothing but the banded factorization and substitution reads W (the
+// explicit inverse reads all of the lower triangle)
+static rbf_status to_f32(const double* H, int64_t ldh, int64_t n, float* W, int64_t ldw, cudaStream_t s, int64_t bw,
+                         bool band_only) {
   int64_t tot = n * n;
+  const int64_t below = bw + 191;
+  if (band_only && below + 128 < n && n <= 65535) {
+    dim3 g((unsigned)((below + 128 + 255) / 256), (unsigned)n);
+    { k_mx_to_f32_band<<<g, 256, 0, s>>>(H, ldh, n, below, W, ldw); ::rbf::note_launch(); }
+    RBF_CUDA(cudaGetLastError());
+    return RBF_OK;
+  }
   { k_mx_to_f32<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(H, ldh, n, W, ldw); ::rbf::note_launch(); }
   RBF_CUDA(cudaGetLastError());
   return RBF_OK;
@@ -568,33 +589,34 @@ static rbf_status to_f32(const double* H, int64_t ldh, int64_t n, float* W, int6
 rbf_status potrf_mixed(Ctx* c, const double* H, int64_t ldh, int64_t n, float* W, int64_t ldw, float* Zd,
                        cudaStream_t s, int64_t bw) {
   if (n <= 0) return RBF_OK;
+  const bool band_only = n > c->inv_max && bw < n;
   cudaStreamCaptureStatus cap0 = cudaStreamCaptureStatusNone;
   RBF_CUDA(cudaStreamIsCapturing(s, &cap0));
   if (!(c->la_ok && c->df_ok && n <= DF_NMAX && cap0 == cudaStreamCaptureStatusNone)) {
-    RBF_TRY(to_f32(H, ldh, n, W, ldw, s));
+    RBF_TRY(to_f32(H, ldh, n, W, ldw, s, bw, band_only));
     return potrf_chain(c, n, W, ldw, Zd, s, bw);
   }
   const int b = (int)(n / 256);
   int8_t& pick = c->fchoice[b < 64 ? b : 63];
   if (pick == 1) {
-    RBF_TRY(to_f32(H, ldh, n, W, ldw, s));
+    RBF_TRY(to_f32(H, ldh, n, W, ldw, s, bw, band_only));
     return potrf_chain(c, n, W, ldw, Zd, s, bw);
   }
   if (pick == 2) {
-    RBF_TRY(to_f32(H, ldh, n, W, ldw, s));
+    RBF_TRY(to_f32(H, ldh, n, W, ldw, s, bw, band_only));
     rbf_status st = potrf_df(c, n, W, ldw, Zd, s, bw);
     if (st != RBF_ERANGE) return st;
-    RBF_TRY(to_f32(H, ldh, n, W, ldw, s));
+    RBF_TRY(to_f32(H, ldh, n, W, ldw, s, bw, band_only));
     return potrf_chain(c, n, W, ldw, Zd, s, bw);
   }
   // first block of this size: time both (the dataflow result is kept)
   cudaEvent_t ev[3];
   for (auto& e : ev) RBF_CUDA(cudaEventCreate(&e));
   RBF_CUDA(cudaEventRecord(ev[0], s));
-  RBF_TRY(to_f32(H, ldh, n, W, ldw, s));
+  RBF_TRY(to_f32(H, ldh, n, W, ldw, s, bw, band_only));
   RBF_TRY(potrf_chain(c, n, W, ldw, Zd, s, bw));
   RBF_CUDA(cudaEventRecord(ev[1], s));
-  RBF_TRY(to_f32(H, ldh, n, W, ldw, s));
+  RBF_TRY(to_f32(H, ldh, n, W, ldw, s, bw, band_only));
   rbf_status st = potrf_df(c, n, W, ldw, Zd, s, bw);
   RBF_CUDA(cudaEventRecord(ev[2], s));
   RBF_CUDA(cudaEventSynchronize(ev[2]));
@@ -604,7 +626,7 @@ rbf_status potrf_mixed(Ctx* c, const double* H, int64_t ldh, int64_t n, float* W
   for (auto& e : ev) cudaEventDestroy(e);
   if (st == RBF_ERANGE) {
     pick = 1;
-    RBF_TRY(to_f32(H, ldh, n, W, ldw, s));
+    RBF_TRY(to_f32(H, ldh, n, W, ldw, s, bw, band_only));
     return potrf_chain(c, n, W, ldw, Zd, s, bw);
   }
   RBF_TRY(st);
@@ -841,17 +863,18 @@ __global__ void k_add_f32_to_f64(double* __restrict__ x, const float* __restrict
 
 // R = B - H X for m right-hand sides (row-major n x m): one warp per row of H,
 // 8 right-hand sides per pass, lanes stride over the row.
-__global__ void __launch_bounds__(256) k_residual_multi(const double* __restrict__ H, int64_t n, int64_t ldh,
+__global__ void __launch_bounds__(256) k_residual_multi(const double* __restrict__ H, int64_t n, int64_t ldh, int64_t bw,
                                                         const double* __restrict__ X, const double* __restrict__ Bm,
                                                         int64_t m, double* __restrict__ R) {
   int lane = threadIdx.x & 31;
   int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (row >= n) return;
   const double* hr = H + row * ldh;
+  const int64_t t0 = row > bw ? row - bw : 0, t1 = row + bw < n ? row + bw + 1 : n;
   for (int64_t j0 = 0; j0 < m; j0 += 8) {
     int q = (int)((m - j0) < 8 ? (m - j0) : 8);
     double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int64_t t = lane; t < n; t += 32) {
+    for (int64_t t = t0 + lane; t < t1; t += 32) {
       double h = hr[t];
       const double* xr = X + t * m + j0;
 #pragma unroll
@@ -909,10 +932,10 @@ rbf_status mixed_solve(Ctx* c, const double* H, int64_t ldh, const SpH* Hs, cons
       if (Hs) {
         RBF_TRY(csr_residual(*Hs, X, bb.as<double>(), m, Rr, s));
       } else if (m == 1) {
-        RBF_TRY(symv_residual(H, n, ldh, X, bb.as<double>(), Rr, s));
+        RBF_TRY(symv_residual(H, n, ldh, X, bb.as<double>(), Rr, s, bw));
       } else {
         unsigned nw = (unsigned)((n * 32 + 255) / 256);
-        { k_residual_multi<<<nw, 256, 0, s>>>(H, n, ldh, X, bb.as<double>(), m, Rr); ::rbf::note_launch(); }
+        { k_residual_multi<<<nw, 256, 0, s>>>(H, n, ldh, bw, X, bb.as<double>(), m, Rr); ::rbf::note_launch(); }
         RBF_CUDA(cudaGetLastError());
       }
       R = Rr;
@@ -983,7 +1006,7 @@ rbf_status mixed_cov(Ctx* c, const double* H, int64_t ldh, const SpH* Hs, const 
     RBF_TRY(csr_residual_ff(c, *Hs, B, e0.as<double>(), k, R, s, 97));
   } else {
     unsigned nw = (unsigned)((n * 32 + 255) / 256);
-    { k_residual_multi<<<nw, 256, 0, s>>>(H, n, ldh, B, e0.as<double>(), k, R); ::rbf::note_launch(); }
+    { k_residual_multi<<<nw, 256, 0, s>>>(H, n, ldh, bw, B, e0.as<double>(), k, R); ::rbf::note_launch(); }
     RBF_CUDA(cudaGetLastError());
   }
   Buf& gq = c->scratch(86);

@@ -20,7 +20,7 @@ namespace {
 // nonzeros per row (one warp per row)
 // nonzeros per row (one warp per row) and the half-bandwidth max |i - j|
 // over the nonzero entries (atomicMax into *bw)
-__global__ void __launch_bounds__(256) k_csr_count(const double* __restrict__ H, int64_t n, int64_t ld,
+__global__ void __launch_bounds__(256) k_csr_count(const double* __restrict__ H, int64_t n, int64_t ld, int64_t band,
                                                    int32_t* __restrict__ cnt, int* __restrict__ bw) {
   const int lane = threadIdx.x & 31;
   const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -28,9 +28,10 @@ __global__ void __launch_bounds__(256) k_csr_count(const double* __restrict__ H,
   const double* hr = H + row * ld;
   int c = 0;
   int64_t far = 0;
-  for (int64_t j0 = 0; j0 < n; j0 += 32) {
+  const int64_t j1 = row + band < n ? row + band + 1 : n;
+  for (int64_t j0 = row > band ? row - band : 0; j0 < j1; j0 += 32) {
     int64_t j = j0 + lane;
-    bool nz = j < n && hr[j] != 0.0;
+    bool nz = j < j1 && hr[j] != 0.0;
     c += __popc(__ballot_sync(0xffffffffu, nz));
     if (nz) {
       int64_t dj = j > row ? j - row : row - j;
@@ -49,7 +50,7 @@ __global__ void __launch_bounds__(256) k_csr_count(const double* __restrict__ H,
 }
 
 // column indices and values in ascending column order (one warp per row)
-__global__ void __launch_bounds__(256) k_csr_fill(const double* __restrict__ H, int64_t n, int64_t ld,
+__global__ void __launch_bounds__(256) k_csr_fill(const double* __restrict__ H, int64_t n, int64_t ld, int64_t band,
                                                   const int32_t* __restrict__ rp, int32_t* __restrict__ col,
                                                   double* __restrict__ val) {
   const int lane = threadIdx.x & 31;
@@ -58,9 +59,10 @@ __global__ void __launch_bounds__(256) k_csr_fill(const double* __restrict__ H, 
   const double* hr = H + row * ld;
   int base = rp[row];
   const unsigned below = (1u << lane) - 1u;
-  for (int64_t j0 = 0; j0 < n; j0 += 32) {
+  const int64_t j1 = row + band < n ? row + band + 1 : n;
+  for (int64_t j0 = row > band ? row - band : 0; j0 < j1; j0 += 32) {
     int64_t j = j0 + lane;
-    double v = j < n ? hr[j] : 0.0;
+    double v = j < j1 ? hr[j] : 0.0;
     bool nz = v != 0.0;
     unsigned m = __ballot_sync(0xffffffffu, nz);
     if (nz) {
@@ -139,8 +141,9 @@ unsigned warps_grid(int64_t n) { return (unsigned)((n * 32 + 255) / 256); }
 
 }  // namespace
 
+// band: a bound of the half-bandwidth; only that part of H is read.
 // The half-bandwidth is left in scratch slot 70 at index n (read by csr_bandwidth).
-rbf_status build_csr(Ctx* c, const double* H, int64_t ld, int64_t n, SpH& out, cudaStream_t s) {
+rbf_status build_csr(Ctx* c, const double* H, int64_t ld, int64_t n, int64_t band, SpH& out, cudaStream_t s) {
   out.valid = false;
   out.n = n;
   if (n <= 0 || n > SPH_MAX) return RBF_OK;
@@ -150,10 +153,10 @@ rbf_status build_csr(Ctx* c, const double* H, int64_t ld, int64_t n, SpH& out, c
   Buf& cnt = c->scratch(70);
   RBF_TRY(cnt.ensure((size_t)(n + 1) * sizeof(int32_t)));
   RBF_CUDA(cudaMemsetAsync(cnt.as<int32_t>() + n, 0, sizeof(int32_t), s));
-  { k_csr_count<<<warps_grid(n), 256, 0, s>>>(H, n, ld, cnt.as<int32_t>(), cnt.as<int32_t>() + n); ::rbf::note_launch(); }
+  { k_csr_count<<<warps_grid(n), 256, 0, s>>>(H, n, ld, band, cnt.as<int32_t>(), cnt.as<int32_t>() + n); ::rbf::note_launch(); }
   RBF_CUDA(cudaGetLastError());
   RBF_TRY(scan_i32(c, cnt.as<int32_t>(), out.rp.as<int32_t>(), n, s, 71));
-  { k_csr_fill<<<warps_grid(n), 256, 0, s>>>(H, n, ld, out.rp.as<int32_t>(), out.col.as<int32_t>(),
+  { k_csr_fill<<<warps_grid(n), 256, 0, s>>>(H, n, ld, band, out.rp.as<int32_t>(), out.col.as<int32_t>(),
                                              out.val.as<double>()); ::rbf::note_launch(); }
   RBF_CUDA(cudaGetLastError());
   out.valid = true;
@@ -174,7 +177,7 @@ rbf_status dense_bandwidth(Ctx* c, const double* H, int64_t ld, int64_t n, int64
   Buf& cnt = c->scratch(70);
   RBF_TRY(cnt.ensure((size_t)(n + 1) * sizeof(int32_t)));
   RBF_CUDA(cudaMemsetAsync(cnt.as<int32_t>() + n, 0, sizeof(int32_t), s));
-  { k_csr_count<<<warps_grid(n), 256, 0, s>>>(H, n, ld, cnt.as<int32_t>(), cnt.as<int32_t>() + n); ::rbf::note_launch(); }
+  { k_csr_count<<<warps_grid(n), 256, 0, s>>>(H, n, ld, BW_DENSE, cnt.as<int32_t>(), cnt.as<int32_t>() + n); ::rbf::note_launch(); }
   RBF_CUDA(cudaGetLastError());
   return csr_bandwidth(c, n, bw, s);
 }
