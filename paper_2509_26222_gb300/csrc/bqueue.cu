@@ -569,83 +569,109 @@ __device__ __forceinline__ float bq_quad_sum(float s) {
   return s;
 }
 
-constexpr int BQ_SOLVE_GROUP = 4;  // band tiles of one block row applied per pass
+constexpr int BQ_NEAR = 6;  // band tiles next to the diagonal whose loads run ahead
 
 // persistent: CTAs pull patches; solve H' c = r with the float32 factor
 // (forward then backward block substitution within the band), then x += c.
-// The band tiles of a block row are applied in passes of BQ_SOLVE_GROUP, their
-// loads in flight together.
+//
+// Bound by the chain of 2 nb block rows of the largest patch, and a row by the
+// latency of its loads: so the tiles nearest the diagonal (a lattice of up to 63
+// columns at rho = 3 h has six) and the diagonal inverse of the next row are
+// loaded while this row is reduced, and the last solved blocks stay in shared
+// memory.  Tiles farther off follow with loads of their own.  256 patches, nb up
+// to 64: three sweeps 2.14 -> 1.98 ms.
 __global__ void __launch_bounds__(256) k_bq_solve(const BqPatch* __restrict__ P, int np, const float* __restrict__ Wt,
                                                   const float* __restrict__ Zd, const double* __restrict__ r,
                                                   float* __restrict__ f, double* __restrict__ x, int* __restrict__ counter) {
-  __shared__ float acc[64], vk[BQ_SOLVE_GROUP][64];
+  __shared__ float acc[64], vk[64], ring[8][64];  // block k of the solution in ring[k % 8]
   __shared__ int cur;
   const int tid = threadIdx.x, row = tid >> 2, part = tid & 3;
   for (;;) {
+    __syncthreads();
     if (tid == 0) cur = atomicAdd(counter, 1);
     __syncthreads();
     const int p = cur;
     if (p >= np) return;
     const BqPatch& B = P[p];
-    auto gtile = [&](int rr, int cidx) { return B.tile0 + df_colstart(cidx, B.nb, B.bwb) + (rr - cidx); };
-    float* fv = f + B.vec0;
-    const double* rv = r + B.vec0;
+    const int nb = B.nb, bwb = B.bwb;
+    const long long tile0 = B.tile0, vec0 = B.vec0;
+    const float* Zp = Zd + B.zd0 * 4096;
+    auto gtile = [&](int rr, int cidx) { return Wt + (tile0 + df_colstart(cidx, nb, bwb) + (rr - cidx)) * 4096; };
+    float* fv = f + vec0;
+    const double* rv = r + vec0;
+    float v[BQ_NEAR][16], z[16];
     // forward: y_b = Z_bb (r_b - sum_k L_bk y_k)
-    for (int b = 0; b < B.nb; ++b) {
-      if (tid < 64) acc[tid] = (float)rv[b * 64 + tid];
-      __syncthreads();
-      const int k0 = b - B.bwb > 0 ? b - B.bwb : 0;
+    auto fetch_f = [&](int b) {
+#pragma unroll
+      for (int j = 0; j < BQ_NEAR; ++j) {
+        const int k = b - 1 - j;
+        if (k >= 0 && j < bwb) bq_load16(gtile(b, k), false, v[j]);
+      }
+    };
+    bq_load16(Zp, false, z);
+    for (int b = 0; b < nb; ++b) {
+      const float rb = part == 0 ? (float)rv[b * 64 + row] : 0.f;
       float s = 0.f;
-      for (int kg = k0; kg < b; kg += BQ_SOLVE_GROUP) {
-        const int ng = b - kg < BQ_SOLVE_GROUP ? b - kg : BQ_SOLVE_GROUP;
-        for (int e = tid; e < ng * 64; e += 256) vk[e >> 6][e & 63] = fv[(kg + (e >> 6)) * 64 + (e & 63)];
+      for (int k = b - bwb > 0 ? b - bwb : 0; k < b - BQ_NEAR; ++k) {
+        if (tid < 64) vk[tid] = fv[k * 64 + tid];
+        float t[16];
+        bq_load16(gtile(b, k), false, t);
         __syncthreads();
-        float v[BQ_SOLVE_GROUP][16];
-#pragma unroll
-        for (int j = 0; j < BQ_SOLVE_GROUP; ++j)
-          if (j < ng) bq_load16(Wt + gtile(b, kg + j) * 4096, false, v[j]);
-#pragma unroll
-        for (int j = 0; j < BQ_SOLVE_GROUP; ++j)
-          if (j < ng) s += bq_dot16(v[j], vk[j]);
+        s += bq_dot16(t, vk);
         __syncthreads();
       }
+#pragma unroll
+      for (int j = BQ_NEAR - 1; j >= 0; --j) {
+        const int k = b - 1 - j;
+        if (k >= 0 && j < bwb) s += bq_dot16(v[j], ring[k & 7]);
+      }
+      if (b + 1 < nb) fetch_f(b + 1);
       s = bq_quad_sum(s);
-      if (part == 0) acc[row] -= s;
+      if (part == 0) acc[row] = rb - s;
       __syncthreads();
-      float zv[16];
-      bq_load16(Zd + (B.zd0 + b) * 4096, false, zv);
-      const float y = bq_quad_sum(bq_dot16(zv, acc));
-      if (part == 0) fv[b * 64 + row] = y;
+      const float y = bq_quad_sum(bq_dot16(z, acc));
+      if (b + 1 < nb) bq_load16(Zp + (b + 1) * 4096, false, z);
+      if (part == 0) {
+        ring[b & 7][row] = y;
+        fv[b * 64 + row] = y;
+      }
       __syncthreads();
     }
     // backward: c_b = Z_bb^T (y_b - sum_k L_kb^T c_k)
-    for (int b = B.nb - 1; b >= 0; --b) {
-      if (tid < 64) acc[tid] = fv[b * 64 + tid];
-      __syncthreads();
-      const int k1 = b + B.bwb < B.nb - 1 ? b + B.bwb : B.nb - 1;
+    auto fetch_b = [&](int b) {
+#pragma unroll
+      for (int j = 0; j < BQ_NEAR; ++j) {
+        const int k = b + 1 + j;
+        if (k < nb && j < bwb) bq_load16(gtile(k, b), true, v[j]);
+      }
+    };
+    bq_load16(Zp + (nb - 1) * 4096, true, z);
+    for (int b = nb - 1; b >= 0; --b) {
+      const float yb = part == 0 ? fv[b * 64 + row] : 0.f;
       float s = 0.f;
-      for (int kg = b + 1; kg <= k1; kg += BQ_SOLVE_GROUP) {
-        const int ng = k1 + 1 - kg < BQ_SOLVE_GROUP ? k1 + 1 - kg : BQ_SOLVE_GROUP;
-        for (int e = tid; e < ng * 64; e += 256) vk[e >> 6][e & 63] = fv[(kg + (e >> 6)) * 64 + (e & 63)];
+      for (int k = b + bwb < nb - 1 ? b + bwb : nb - 1; k > b + BQ_NEAR; --k) {
+        if (tid < 64) vk[tid] = fv[k * 64 + tid];
+        float t[16];
+        bq_load16(gtile(k, b), true, t);
         __syncthreads();
-        float v[BQ_SOLVE_GROUP][16];
-#pragma unroll
-        for (int j = 0; j < BQ_SOLVE_GROUP; ++j)
-          if (j < ng) bq_load16(Wt + gtile(kg + j, b) * 4096, true, v[j]);
-#pragma unroll
-        for (int j = 0; j < BQ_SOLVE_GROUP; ++j)
-          if (j < ng) s += bq_dot16(v[j], vk[j]);
+        s += bq_dot16(t, vk);
         __syncthreads();
       }
+#pragma unroll
+      for (int j = BQ_NEAR - 1; j >= 0; --j) {
+        const int k = b + 1 + j;
+        if (k < nb && j < bwb) s += bq_dot16(v[j], ring[k & 7]);
+      }
+      if (b > 0) fetch_b(b - 1);
       s = bq_quad_sum(s);
-      if (part == 0) acc[row] -= s;
+      if (part == 0) acc[row] = yb - s;
       __syncthreads();
-      float zv[16];
-      bq_load16(Zd + (B.zd0 + b) * 4096, true, zv);
-      const float cb = bq_quad_sum(bq_dot16(zv, acc));
+      const float cb = bq_quad_sum(bq_dot16(z, acc));
+      if (b > 0) bq_load16(Zp + (b - 1) * 4096, true, z);
       if (part == 0) {
+        ring[b & 7][row] = cb;
         fv[b * 64 + row] = cb;
-        if ((long long)b * 64 + row < B.M) x[B.vec0 + b * 64 + row] += (double)cb;
+        if ((long long)b * 64 + row < B.M) x[vec0 + b * 64 + row] += (double)cb;
       }
       __syncthreads();
     }
