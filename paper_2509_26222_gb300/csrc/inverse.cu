@@ -19,6 +19,7 @@
 #include <cuda_runtime.h>
 
 #include "common.cuh"
+#include "tc_util.cuh"
 
 namespace rbf {
 namespace {
@@ -173,6 +174,201 @@ __global__ void __launch_bounds__(256) k_trtri_level(int kind, int64_t b, int64_
   }
 }
 
+// The same products for the levels whose half has TT_MIN rows or more, on the
+// tensor cores: one 128 x 128 tile of the output per CTA (or half of its K
+// range), C = A B with float32 operands split into three bfloat16 slices on
+// their way into shared memory and the six slice products down to 2^-24 of
+// |A| |B| accumulated in float32 in tensor memory, as in the trailing update.
+//
+// The large levels are nearly all of the n^3 / 3 multiply-adds.  On the float32 pipe 64 x 64 tiles reach 16 to 20 TFLOP/s there,
+// bound by their shared-memory loads.  Here a chunk of K = 64 costs a CTA 24
+// instructions of 128 x 128 x 16 and the split of 2 x 8,192 floats; two CTAs on
+// an SM overlap the two.  B comes as rows of K, so a thread splits two
+// neighbouring rows and stores pairs, which makes B K-major.
+// Whole inverse: a = 3,750: 893 -> 459 us; a = 2,500: 513 -> 298; a = 1,807:
+// 176 -> 146.  At half-size 512 (a = 1,807 and 3,750) this kernel takes 48 and
+// 52 us for the two products, the float32 tiles 41 and 58: the line is at 1024.
+constexpr int TT_MIN = 1024;
+constexpr int TT_K = 64;
+constexpr int TT_SLICE = 128 * TT_K * 2;             // bytes of a 128 x 64 bf16 slice
+constexpr int TT_SMEM = 6 * TT_SLICE + 1024;
+
+// x and y as three bfloat16 each (24 bits, every slice rounded to nearest), slice
+// t of x in the low and of y in the high half of q[t].  The rounding is an integer
+// addition: the conversion instruction runs at a fraction of the rate.
+__device__ __forceinline__ void split3(float x, float y, uint32_t (&q)[3]) {
+#pragma unroll
+  for (int t = 0; t < 3; ++t) {
+    const uint32_t a = (__float_as_uint(x) + 0x8000u) & 0xffff0000u, b = (__float_as_uint(y) + 0x8000u) & 0xffff0000u;
+    q[t] = __byte_perm(a, b, 0x7632);
+    x -= __uint_as_float(a);
+    y -= __uint_as_float(b);
+  }
+}
+
+__global__ void __launch_bounds__(256, 2) k_trtri_tc(int kind, int64_t b, int64_t n, const float* __restrict__ W,
+                                                     int64_t ldw, float* __restrict__ Z, int64_t ldz,
+                                                     float* __restrict__ T, int split, int* __restrict__ status) {
+  extern __shared__ uint8_t tt_raw[];
+  __shared__ uint64_t mbar;
+  __shared__ uint32_t tmem_slot;
+  __shared__ int ok_s;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t p = split == 2 ? (blockIdx.z >> 1) : blockIdx.z;
+  const int64_t r1 = p * b, h1 = b / 2, r2 = r1 + h1;
+  const int64_t h2 = (n - r2) < h1 ? (n - r2) : h1;
+  const int64_t i0 = (int64_t)blockIdx.y * 128, j0 = (int64_t)blockIdx.x * 128;
+  if (h2 <= 0 || i0 >= h2 || j0 >= h1) return;
+  // K range: kind 0 T21 = L21 Z11 (Z11 lower: k >= j0), kind 1 Z21 = -Z22 T21 (Z22 lower: k < i0 + 128)
+  int64_t kb = kind == 0 ? j0 : 0;
+  const int64_t kn = kind == 0 ? h1 : h2;  // rows of B
+  int64_t ke = kind == 0 ? h1 : ((i0 + 128) < h2 ? (i0 + 128) : h2);
+  if (split == 2) {
+    int64_t mid = kb + ((ke - kb) / 2 + TT_K - 1) / TT_K * TT_K;
+    if (mid > ke) mid = ke;
+    if (blockIdx.z & 1) kb = mid;
+    else ke = mid;
+  }
+  if (kb >= ke) return;
+  const float* A = kind == 0 ? W + r2 * ldw + r1 : Z + r2 * ldz + r2;
+  const int64_t lda = kind == 0 ? ldw : ldz;
+  const float* B = kind == 0 ? Z + r1 * ldz + r1 : T + r2 * ldz + r1;
+  float* C = (kind == 0 ? T : Z) + r2 * ldz + r1;
+  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(tt_raw) + 1023) & ~(uintptr_t)1023);
+  if (warp == 0) tc::tmem_alloc(&tmem_slot, 128);
+  if (tid == 0) tc::mbar_init(&mbar, 1);
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  const uint32_t tmem = tmem_slot;
+  // A: rows tid / 16 + 16 q, 4 columns from 4 (tid % 16); B: row pairs 4 (warp % 8) + lane / 8, 4 columns from
+  // 32 q + 4 (lane % 8): whole 128-byte lines in every load
+  const int ar = tid >> 4, ac = (tid & 15) * 4;
+  const int kp = 4 * warp + (lane >> 3), jl = lane & 7;
+  float4 av[8], b0[4], b1[4];
+  auto fetch = [&](int64_t k0) {
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float* pa = A + (i0 + ar) * lda + k0 + ac;
+    // (columns past the matrix but inside the padded row hold zeros or are times a zero row of B)
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      av[q] = (i0 + ar + 16 * q < h2 && k0 + ac < kn) ? *reinterpret_cast<const float4*>(pa + 16 * q * lda) : zero;
+    const int64_t k = k0 + 2 * kp;
+    const float* pb = B + k * ldz + j0 + 4 * jl;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      b0[q] = k < kn ? *reinterpret_cast<const float4*>(pb + 32 * q) : zero;
+      b1[q] = k + 1 < kn ? *reinterpret_cast<const float4*>(pb + ldz + 32 * q) : zero;
+    }
+  };
+  // component (e + jl / 2) % 4 first: the eight lanes of a row pair then store to
+  // rows of eight different swizzle phases, so that a warp's stores meet 32 banks
+  auto rotated = [&](const float4& v, float (&x)[4]) {
+    const bool r1 = (jl >> 1) & 1, r2 = (jl >> 2) & 1;
+    const float t[4] = {r1 ? v.y : v.x, r1 ? v.z : v.y, r1 ? v.w : v.z, r1 ? v.x : v.w};
+    x[0] = r2 ? t[2] : t[0];
+    x[1] = r2 ? t[3] : t[1];
+    x[2] = r2 ? t[0] : t[2];
+    x[3] = r2 ? t[1] : t[3];
+  };
+  uint32_t phase = 0;
+  bool ok = true;
+  auto wait = [&]() {  // the products of the last chunk
+    if (tid == 0) {
+      long long it = 0;
+      bool got;
+      while (!(got = tc::mbar_try_wait(&mbar, phase)) && ++it < tc::WAIT_LIMIT) {
+      }
+      if (!got) {
+        atomicOr(status, DEV_TIMEOUT);
+        // one more bounded chance to drain before the operands and TMEM are given back
+        for (it = 0; !tc::mbar_try_wait(&mbar, phase) && it < tc::WAIT_LIMIT; ++it) {
+        }
+      }
+      ok_s = got ? 1 : 0;
+    }
+    __syncthreads();
+    tc::fence_after();
+    ok = ok_s != 0;
+    phase ^= 1;
+  };
+  fetch(kb);
+  for (int64_t k0 = kb; k0 < ke && ok; k0 += TT_K) {
+    if (k0 > kb) wait();
+    if (!ok) break;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      uint32_t lo[3], hi[3];
+      split3(av[q].x, av[q].y, lo);
+      split3(av[q].z, av[q].w, hi);
+      const uint32_t off = tc::sw128_offset(ar + 16 * q, ac >> 3) + 2 * (ac & 7);
+#pragma unroll
+      for (int t = 0; t < 3; ++t)
+        *reinterpret_cast<uint2*>(sm + t * TT_SLICE + off) = make_uint2(lo[t], hi[t]);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float x[4], y[4];
+      rotated(b0[q], x);
+      rotated(b1[q], y);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        uint32_t w[3];
+        split3(x[e], y[e], w);
+        const int j = 32 * q + 4 * jl + ((e + (jl >> 1)) & 3);
+        const uint32_t off = tc::sw128_offset(j, kp >> 2) + 4 * (kp & 3);
+#pragma unroll
+        for (int t = 0; t < 3; ++t)
+          *reinterpret_cast<uint32_t*>(sm + (3 + t) * TT_SLICE + off) = w[t];
+      }
+    }
+    tc::fence_proxy_async();
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+    if (tid == 0) {
+      const int pa[6] = {0, 0, 1, 0, 1, 2}, pb[6] = {0, 1, 0, 2, 1, 0};
+#pragma unroll
+      for (int q = 0; q < 6; ++q) {
+        const uint64_t ad = tc::sdesc_sw128(tc::smem_u32(sm + pa[q] * TT_SLICE));
+        const uint64_t bd = tc::sdesc_sw128(tc::smem_u32(sm + (3 + pb[q]) * TT_SLICE));
+#pragma unroll
+        for (int kk = 0; kk < TT_K / 16; ++kk)
+          tc::mma_bf16(tmem, ad + (uint64_t)(2 * kk), bd + (uint64_t)(2 * kk), (k0 > kb || q > 0 || kk > 0) ? 1u : 0u);
+      }
+      tc::mma_commit(&mbar);
+    }
+    if (k0 + TT_K < ke) fetch(k0 + TT_K);
+  }
+  if (ok) wait();
+  // epilogue: warp w reads TMEM lanes 32 (w % 4) .., columns 64 (w / 4) .. + 63
+  if (ok) {
+    const int64_t row = i0 + 32 * (warp & 3) + lane;
+    const float alpha = kind == 0 ? 1.f : -1.f;
+#pragma unroll 1
+    for (int cb = 0; cb < 2; ++cb) {
+      const int col = 64 * (warp >> 2) + 32 * cb;
+      float v[32];
+      tc::tmem_ld32(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)col, v);
+      if (row < h2) {
+        float* cr = C + row * ldz + j0 + col;
+        if (split == 2) {
+#pragma unroll
+          for (int e = 0; e < 32; ++e) atomicAdd(cr + e, alpha * v[e]);
+        } else {
+#pragma unroll
+          for (int e = 0; e < 32; e += 4)
+            *reinterpret_cast<float4*>(cr + e) =
+                make_float4(alpha * v[e], alpha * v[e + 1], alpha * v[e + 2], alpha * v[e + 3]);
+        }
+      }
+    }
+  }
+  tc::fence_before();
+  __syncthreads();
+  if (warp == 0) tc::tmem_dealloc(tmem, 128);
+}
+
 // Y = Z F (forward, Z lower) or Y = Zt F (backward, Zt = Z^T upper) for
 // m > GEMV_M right-hand sides; F, Y row-major n x m.  blockIdx.z splits K; partial
 // products go to P[z] and are summed by k_sum_partials.
@@ -308,6 +504,22 @@ rbf_status trtri_mixed(Ctx* c, const float* W, int64_t ldw, int64_t n, const flo
   RBF_CUDA(cudaGetLastError());
   for (int64_t b = 128; b / 2 < n; b *= 2) {
     int64_t h = b / 2;
+    if (h >= TT_MIN) {
+      static bool attr[64] = {false};
+      if (!attr[c->device & 63]) {
+        RBF_CUDA(cudaFuncSetAttribute(k_trtri_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, TT_SMEM));
+        attr[c->device & 63] = true;
+      }
+      // fewer tiles than two per SM: K in two halves (0 + a + b = 0 + b + a exactly)
+      const int64_t tt = (int64_t)cdiv(h, 128) * cdiv(h, 128) * cdiv(n, b);
+      const int sp = tt < 2 * 152 ? 2 : 1;
+      for (int kind = 0; kind < 2; ++kind) {
+        { k_trtri_tc<<<dim3(cdiv(h, 128), cdiv(h, 128), (unsigned)(cdiv(n, b) * sp)), 256, TT_SMEM, s>>>(
+            kind, b, n, W, ldw, Z, ldz, T, sp, c->dflag.as<int>()); ::rbf::note_launch(); }
+        RBF_CUDA(cudaGetLastError());
+      }
+      continue;
+    }
     // levels whose tiles do not fill the GPU twice split K in two halves
     const int64_t tiles = (int64_t)cdiv(h, TG) * cdiv(h, TG) * cdiv(n, b);
     const int split = (tiles < 2 * 152 && h >= 256) ? 2 : 1;

@@ -23,22 +23,9 @@
 namespace rbf {
 namespace tc {
 
-constexpr int TILE = 128;             // M = N = 128
 constexpr int KB = 64;                // panel width (bf16 elements per row)
 constexpr int SLICE_BYTES = TILE * KB * 2;   // 16 KiB per operand slice tile
 constexpr int SMEM_BYTES = 6 * SLICE_BYTES + 1024;  // 3 A + 3 B slices, 1 KiB alignment slack
-// Instruction descriptor: kind::f16, A = B = bf16, D = f32, K-major A and B,
-// N = 128 (bits 17-22: N >> 3), M = 128 (bits 24-28: M >> 4).
-constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TILE >> 3) << 17) |
-                           ((uint32_t)(TILE >> 4) << 24);
-
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accum) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %3, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %4, p;\n\t}\n" ::"r"(tmem_d),
-      "l"(adesc), "l"(bdesc), "r"(accum), "r"(IDESC));
-}
 
 // Copy rows [r0, r0 + 128) of a bf16 slice (row-major, KB elements per row,
 // rows >= m read as zero) into a swizzled tile with asynchronous 16-byte
