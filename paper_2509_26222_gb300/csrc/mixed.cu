@@ -26,22 +26,17 @@
 namespace rbf {
 
 
-__global__ void k_mx_to_f32(const double* __restrict__ H, int64_t ldh, int64_t n, float* __restrict__ W,
-                            int64_t ldw) {
-  int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n * n) return;
-  int64_t i = e / n, j = e % n;
-  W[i * ldw + j] = (float)H[i * ldh + j];
-}
-
-// The same for the part of a banded H that the factorization and the solves
-// read: columns [i - bw - 191, i + 127] (whole 64 x 64 tiles up to two block
-// columns past the band, and the diagonal tile of a 128-wide update).
-// a = 8,189, bw = 390: 235 -> 30 us.
-__global__ void k_mx_to_f32_band(const double* __restrict__ H, int64_t ldh, int64_t n, int64_t below,
-                                 float* __restrict__ W, int64_t ldw) {
-  const int64_t i = blockIdx.y, j = i - below + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (j < 0 || j >= n || j > i + 127) return;
+// The part of H that the factorization, its inverse and the solves read: columns
+// [i - below, i + 127] of row i (the diagonal tile of a 128-wide update), for a
+// banded H with below = bw + 191 (whole 64 x 64 tiles up to two block columns
+// past the band).  All of H is the whole lower triangle and costs half of a full
+// copy: the conversion runs on the float64 pipe.
+// a = 8,189, bw = 390: 235 -> 30 us; a = 3,849, dense: 53 -> 43 us.
+__global__ void k_mx_to_f32(const double* __restrict__ H, int64_t ldh, int64_t n, int64_t i0, int64_t below,
+                            float* __restrict__ W, int64_t ldw) {
+  const int64_t i = i0 + blockIdx.y, first = i > below ? i - below : 0;
+  const int64_t j = first + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= n || j > i + 127) return;
   W[i * ldw + j] = (float)H[i * ldh + j];
 }
 
@@ -567,15 +562,12 @@ static rbf_status potrf_chain(Ctx* c, int64_t n, float* W, int64_t ldw, float* Z
 // explicit inverse reads all of the lower triangle)
 static rbf_status to_f32(const double* H, int64_t ldh, int64_t n, float* W, int64_t ldw, cudaStream_t s, int64_t bw,
                          bool band_only) {
-  int64_t tot = n * n;
-  const int64_t below = bw + 191;
-  if (band_only && below + 128 < n && n <= 65535) {
-    dim3 g((unsigned)((below + 128 + 255) / 256), (unsigned)n);
-    { k_mx_to_f32_band<<<g, 256, 0, s>>>(H, ldh, n, below, W, ldw); ::rbf::note_launch(); }
-    RBF_CUDA(cudaGetLastError());
-    return RBF_OK;
+  const int64_t below = band_only && bw + 191 < n ? bw + 191 : n;
+  const int64_t width = below + 128 < n ? below + 128 : n;
+  for (int64_t i0 = 0; i0 < n; i0 += 65535) {  // rows of one launch (grid limit)
+    const int64_t rows = n - i0 < 65535 ? n - i0 : 65535;
+    { k_mx_to_f32<<<dim3((unsigned)((width + 255) / 256), (unsigned)rows), 256, 0, s>>>(H, ldh, n, i0, below, W, ldw); ::rbf::note_launch(); }
   }
-  { k_mx_to_f32<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(H, ldh, n, W, ldw); ::rbf::note_launch(); }
   RBF_CUDA(cudaGetLastError());
   return RBF_OK;
 }
