@@ -547,6 +547,7 @@ rbf_status reset_update_state(Ctx* c) {
   c->arena_used = 0;
   c->zi_valid = false;
   c->bw_lf = BW_DENSE;
+  c->ends_lf = false;
   c->Hs.valid = false;
   c->Hs_next.valid = false;
   // the outside covariance store keeps its allocation: it is zeroed and set to

@@ -119,6 +119,7 @@ struct Ctx {
   int64_t inv_max = 4096;  // form L^{-1} for active blocks up to this size
   bool gacc_dirty = false; // the Gram accumulators may hold values of an unfinished update
   int64_t bw_lf = BW_DENSE_CTX;  // half-bandwidth of the float32 factor Lf
+  bool ends_lf = false;          // Lf is eliminated from both ends (TwoEnds)
   int64_t nbr_cap = 0;           // neighbour-list capacity of rbf_update (0: read the total first)
   cudaStream_t bs[3] = {};           // side streams of the block stage (bs[2]: high priority)
   cudaEvent_t bev[4] = {};           // fork and joins of the block stage
@@ -301,17 +302,18 @@ rbf_status trsm_lower(Ctx* c, const double* L, int64_t n, int64_t ldl, double* B
 rbf_status gemm_f64(Ctx* c, bool ta, bool tb, int64_t m, int64_t n, int64_t k, double alpha,
                     const double* A, int64_t lda, const double* B, int64_t ldb, double beta,
                     double* Cm, int64_t ldc, cudaStream_t s, int slot = 28);
-// mixed precision (mixed.cu)
+// mixed precision (mixed.cu); ends: the factor is (may be, on return of potrf_mixed)
+// of the rows in the order of TwoEnds
 rbf_status potrf_mixed(Ctx* c, const double* H, int64_t ldh, int64_t n, float* W, int64_t ldw, float* Zd,
-                       cudaStream_t s, int64_t bw = BW_DENSE);
+                       cudaStream_t s, int64_t bw = BW_DENSE, bool* ends = nullptr);
 rbf_status trsm32(Ctx* c, const float* L, int64_t n, int64_t ldl, const float* Zd, float* B, int64_t m,
-                  int64_t ldb, bool transpose, cudaStream_t s, int64_t bw = BW_DENSE);
+                  int64_t ldb, bool transpose, cudaStream_t s, int64_t bw = BW_DENSE, bool ends = false);
 rbf_status mixed_solve(Ctx* c, const double* H, int64_t ldh, const SpH* Hs, const float* W, int64_t ldw,
                        const float* Zd, const float* Zi, int64_t n, double* B, int64_t m, int sweeps,
-                       cudaStream_t s, int64_t bw = BW_DENSE);
+                       cudaStream_t s, int64_t bw = BW_DENSE, bool ends = false);
 rbf_status mixed_cov(Ctx* c, const double* H, int64_t ldh, const SpH* Hs, const float* W, int64_t ldw,
                      const float* Zd, const float* Zi, int64_t n, double* B, int64_t k, const int32_t* pos,
-                     int sweeps, double* P, cudaStream_t s, int64_t bw = BW_DENSE);
+                     int sweeps, double* P, cudaStream_t s, int64_t bw = BW_DENSE, bool ends = false);
 // compressed rows of the information matrix (sparse.cu)
 rbf_status build_csr(Ctx* c, const double* H, int64_t ld, int64_t n, int64_t band, SpH& out, cudaStream_t s);
 rbf_status csr_bandwidth(Ctx* c, int64_t n, int64_t* bw, cudaStream_t s);

@@ -113,6 +113,50 @@ __device__ __forceinline__ int df_colstart(int l, int nb, int bwb) {
   return full * (bwb + 1) + m * s0 - m * (m - 1) / 2;
 }
 
+// Order of the rows of a banded matrix for elimination from both ends.  Block
+// rows of 64 alternate between the top of the matrix, downwards, and its bottom,
+// upwards (rows reversed), so that two independent chains of block columns run
+// side by side and meet in the middle: half the dependent steps of a band.  The
+// last block (the ragged one, if any) is the top's last.  Eliminating a row
+// couples rows within the band only, so tiles farther apart stay zero: `coupled`
+// says which tiles (i, l) of the new order can hold something.  off: the natural
+// order, every tile of the enumerated band.
+struct TwoEnds {
+  int64_t n = 0, bw = 0;
+  int hb = 0, tp = 0;  // blocks from the bottom; parity of the blocks from the top
+  bool on = false;
+  static TwoEnds make(int64_t n, int64_t bw) {
+    TwoEnds t;
+    const int nb = (int)((n + MB - 1) / MB);
+    t.n = n;
+    t.bw = bw;
+    t.hb = nb / 2;
+    t.tp = (nb - 1) & 1;
+    t.on = true;
+    return t;
+  }
+  __device__ __forceinline__ int64_t row_of(int64_t r) const {  // new row of natural row r
+    if (!on) return r;
+    if (r < n - (int64_t)64 * hb) return 64 * (2 * (r >> 6) + tp) + (r & 63);
+    r = n - 1 - r;
+    return 64 * (2 * (r >> 6) + (1 - tp)) + (r & 63);
+  }
+  __device__ __forceinline__ int64_t natural(int64_t r) const {  // natural row of new row r
+    if (!on) return r;
+    const int64_t b = r >> 6, v = 64 * (b >> 1) + (r & 63);
+    return (b & 1) == tp ? v : n - 1 - v;
+  }
+  __device__ __forceinline__ bool coupled(int i, int l) const {
+    if (!on || i == l) return true;
+    const int qi = i >> 1, ql = l >> 1;
+    const int64_t gap = ((i ^ l) & 1) == 0 ? 64 * (int64_t)(qi > ql ? qi - ql : ql - qi) - 63
+                                           : n - 64 * (int64_t)(qi + ql) - 127;
+    return gap <= bw;
+  }
+};
+// tiles below the diagonal that a coupled tile can be away from it (new order)
+inline int two_ends_reach(int64_t bw) { return 2 * (int)((bw + MB - 1) / MB) + 2; }
+
 // k-major staging with the float4 columns xor-swizzled by k: S[kk][r] holds
 // element (r, kk) of a 64 x 64 row-major tile
 __device__ __forceinline__ int df_swz(int kk, int r) { return kk * 64 + (r ^ (((kk >> 2) & 7) << 2)); }

@@ -999,7 +999,7 @@ extern "C" rbf_status rbf_update(rbf_ctx* cx, const float* pts, int64_t n, doubl
       // X = H_prev^{-1} E_D by refined solves with the float32 factor; P_DD = X[D, :]
       RBF_TRY(mixed_cov(c, c->H.as<double>(), c->ldH, &c->Hs, c->Lf.as<float>(), c->ldw, c->Zd.as<float>(),
                         c->zi_valid ? c->Zi.as<float>() : nullptr, ap, Y.as<double>(), d, Dl.as<int32_t>(),
-                        c->refine_sweeps_cov, Pdd.as<double>(), sA, c->bw_lf));
+                        c->refine_sweeps_cov, Pdd.as<double>(), sA, c->bw_lf, c->ends_lf));
     } else {
       // Y = L_prev^{-1} E_D, P_DD = Y^T Y
       RBF_TRY(trsm_lower(c, c->L.as<double>(), ap, c->ldH, Y.as<double>(), d, d, false, s, c->bw_lf));
@@ -1229,10 +1229,11 @@ extern "C" rbf_status rbf_update(rbf_ctx* cx, const float* pts, int64_t n, doubl
   // (the inverse of a banded factor is dense, but for blocks this small the
   // products with it still beat the chain of substitution steps)
   const bool use_inv = mixed && an <= c->inv_max;
+  bool ends = false;  // the factor is eliminated from both ends of the band
   if (mixed) {
     RBF_TRY(Wn.ensure((size_t)an * ldw * sizeof(float)));
     RBF_TRY(Zdn.ensure((size_t)((an + 63) / 64) * 64 * 64 * sizeof(float)));
-    RBF_TRY(potrf_mixed(c, Hn.as<double>(), ld, an, Wn.as<float>(), ldw, Zdn.as<float>(), s, bw));
+    RBF_TRY(potrf_mixed(c, Hn.as<double>(), ld, an, Wn.as<float>(), ldw, Zdn.as<float>(), s, bw, &ends));
     if (use_inv) {
       RBF_TRY(Zin.ensure((size_t)2 * an * ldw * sizeof(float)));  // L^{-1} and its transpose
       RBF_TRY(trtri_mixed(c, Wn.as<float>(), ldw, an, Zdn.as<float>(), Zin.as<float>(), ldw, s));
@@ -1247,7 +1248,7 @@ extern "C" rbf_status rbf_update(rbf_ctx* cx, const float* pts, int64_t n, doubl
                                             (double)an * an);
     if (mixed)
       RBF_TRY(mixed_solve(c, Hn.as<double>(), ld, &c->Hs_next, Wn.as<float>(), ldw, Zdn.as<float>(),
-                          use_inv ? Zin.as<float>() : nullptr, an, u.as<double>(), 1, c->refine_sweeps, s, bw));
+                          use_inv ? Zin.as<float>() : nullptr, an, u.as<double>(), 1, c->refine_sweeps, s, bw, ends));
     else
       RBF_TRY(chol_solve(c, Hn.as<double>(), Ln.as<double>(), an, ld, u.as<double>(), false, s, bw));
   }
@@ -1288,6 +1289,7 @@ extern "C" rbf_status rbf_update(rbf_ctx* cx, const float* pts, int64_t n, doubl
     if (use_inv) std::swap(c->Zi, Zin);
     c->zi_valid = use_inv;
     c->bw_lf = bw;
+    c->ends_lf = ends;
     c->ldw = ldw;
   } else {
     std::swap(c->L, Ln);
@@ -1407,7 +1409,7 @@ extern "C" rbf_status rbf_get_cov(rbf_ctx* cx, const int32_t* ids, int64_t k, do
     if (c->cfg.update_precision == RBF_UPDATE_MIXED) {
       RBF_TRY(mixed_cov(c, c->H.as<double>(), c->ldH, &c->Hs, c->Lf.as<float>(), c->ldw, c->Zd.as<float>(),
                         c->zi_valid ? c->Zi.as<float>() : nullptr, c->a, Y.as<double>(), ka, lb.as<int32_t>(),
-                        c->refine_sweeps_cov, Paa.as<double>(), s, c->bw_lf));
+                        c->refine_sweeps_cov, Paa.as<double>(), s, c->bw_lf, c->ends_lf));
     } else {
       RBF_TRY(trsm_lower(c, c->L.as<double>(), c->a, c->ldH, Y.as<double>(), ka, ka, false, s, c->bw_lf));
       RBF_TRY(gemm_f64(c, true, false, ka, ka, c->a, 1.0, Y.as<double>(), ka, Y.as<double>(), ka, 0.0,
