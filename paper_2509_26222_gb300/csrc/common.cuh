@@ -2,6 +2,8 @@
 #pragma once
 
 #include <cuda_runtime.h>
+
+#include <utility>
 #include <stdint.h>
 
 #include <string>
@@ -288,6 +290,37 @@ inline cudaError_t cooperative_launch(const void* f, dim3 g, dim3 b, void** args
   cudaError_t e = cudaLaunchCooperativeKernel(f, g, b, args, smem, s);
   if (e == cudaSuccess) note_launch();
   return e;
+}
+
+// A launch that may start while the kernel before it on the stream still runs
+// (programmatic dependent launch): its blocks are placed and wait in
+// after_previous() for that kernel's end and writes, instead of coming after it.
+// For chains of short kernels, where the 2 us between two launches count; only
+// for kernels that call after_previous() before they touch global memory.  The
+// call also lets the next such launch be placed.  early = false (stream capture,
+// single launches): an ordinary launch.
+template <class... P, class... A>
+inline cudaError_t launch_early(bool early, void (*f)(P...), dim3 g, dim3 b, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = g;
+  cfg.blockDim = b;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = early ? 1 : 0;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, f, std::forward<A>(args)...);
+  if (e == cudaSuccess) note_launch();
+  return e;
+}
+__device__ __forceinline__ void after_previous() {
+  asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
+}
+inline bool not_capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(s, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone;
 }
 
 // dense FP64 / mixed-precision linear algebra (dense.cu)
