@@ -676,6 +676,7 @@ __global__ void __launch_bounds__(256) k_symv_residual(const double* __restrict_
                                                        const double* __restrict__ x,
                                                        const double* __restrict__ b,
                                                        double* __restrict__ r) {
+  after_previous();
   int lane = threadIdx.x & 31;
   int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (row >= n) return;
@@ -690,8 +691,7 @@ __global__ void __launch_bounds__(256) k_symv_residual(const double* __restrict_
 rbf_status symv_residual(const double* H, int64_t n, int64_t ld, const double* x, const double* b,
                          double* r, cudaStream_t s, int64_t bw) {
   if (n <= 0) return RBF_OK;
-  { k_symv_residual<<<(unsigned)((n * 32 + 255) / 256), 256, 0, s>>>(H, n, ld, bw, x, b, r); ::rbf::note_launch(); }
-  RBF_CUDA(cudaGetLastError());
+  RBF_CUDA(launch_early(not_capturing(s), k_symv_residual, (unsigned)((n * 32 + 255) / 256), 256, 0, s, H, n, ld, bw, x, b, r));
   return RBF_OK;
 }
 

@@ -119,6 +119,7 @@ __device__ __forceinline__ void tile_store(const float (&acc)[4][4], float alpha
 
 // Copy the 64 x 64 diagonal inverses into Z (whose other entries are zero).
 __global__ void k_inv_diag(const float* __restrict__ Zd, int64_t n, float* __restrict__ Z, int64_t ldz) {
+  after_previous();
   int64_t q = blockIdx.x;
   int64_t k = q * 64;
   int kb = (int)((n - k) < 64 ? (n - k) : 64);
@@ -139,6 +140,7 @@ __global__ void __launch_bounds__(256) k_trtri_level(int kind, int64_t b, int64_
                                                      float* __restrict__ T, int split) {
   __shared__ __align__(16) float As[TK][TLD];
   __shared__ __align__(16) float Bs[TK][TLD];
+  after_previous();
   const int64_t p = split == 2 ? (blockIdx.z >> 1) : blockIdx.z;
   const int half = split == 2 ? (int)(blockIdx.z & 1) : -1;
   const int64_t r1 = p * b, h1 = b / 2, r2 = r1 + h1;
@@ -235,6 +237,7 @@ __global__ void __launch_bounds__(256, 2) k_trtri_tc(int kind, int64_t b, int64_
   const float* B = kind == 0 ? Z + r1 * ldz + r1 : T + r2 * ldz + r1;
   float* C = (kind == 0 ? T : Z) + r2 * ldz + r1;
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(tt_raw) + 1023) & ~(uintptr_t)1023);
+  after_previous();
   if (warp == 0) tc::tmem_alloc(&tmem_slot, 128);
   if (tid == 0) tc::mbar_init(&mbar, 1);
   tc::fence_before();
@@ -406,7 +409,8 @@ __global__ void k_sum_partials(const float* __restrict__ P, int nsplit, int64_t 
 template <bool UPPER>
 __global__ void __launch_bounds__(256) k_inv_gemv(int64_t n, int m, const float* __restrict__ A, int64_t lda,
                                                   const float* __restrict__ F, float* __restrict__ Y,
-                                                  double* __restrict__ Xd = nullptr) {
+                                                  double* __restrict__ Xd) {
+  after_previous();
   const int lane = threadIdx.x & 31;
   const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (i >= n) return;
@@ -446,6 +450,7 @@ __global__ void __launch_bounds__(256) k_inv_gemv(int64_t n, int m, const float*
 // Zt = Z^T (n x n, both with leading dimension ld), 32 x 32 tiles
 __global__ void k_transpose32(const float* __restrict__ Z, int64_t n, int64_t ld, float* __restrict__ Zt) {
   __shared__ float t[32][33];
+  after_previous();
   const int64_t bx = (int64_t)blockIdx.x * 32, by = (int64_t)blockIdx.y * 32;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8 threads
   for (int r = ty; r < 32; r += 8) {
@@ -500,8 +505,8 @@ rbf_status trtri_mixed(Ctx* c, const float* W, int64_t ldw, int64_t n, const flo
   StageTimer st(c, RBF_STAGE_INVERSE, s, (double)n * n * n / 3.0);
   RBF_CUDA(cudaMemsetAsync(Z, 0, (size_t)n * ldz * sizeof(float), s));
   RBF_CUDA(cudaMemsetAsync(T, 0, (size_t)n * ldz * sizeof(float), s));  // levels write disjoint blocks
-  { k_inv_diag<<<cdiv(n, 64), 256, 0, s>>>(Zd, n, Z, ldz); ::rbf::note_launch(); }
-  RBF_CUDA(cudaGetLastError());
+  const bool early = not_capturing(s);
+  RBF_CUDA(launch_early(early, k_inv_diag, cdiv(n, 64), 256, 0, s, Zd, n, Z, ldz));
   for (int64_t b = 128; b / 2 < n; b *= 2) {
     int64_t h = b / 2;
     if (h >= TT_MIN) {
@@ -514,9 +519,8 @@ rbf_status trtri_mixed(Ctx* c, const float* W, int64_t ldw, int64_t n, const flo
       const int64_t tt = (int64_t)cdiv(h, 128) * cdiv(h, 128) * cdiv(n, b);
       const int sp = tt < 2 * 152 ? 2 : 1;
       for (int kind = 0; kind < 2; ++kind) {
-        { k_trtri_tc<<<dim3(cdiv(h, 128), cdiv(h, 128), (unsigned)(cdiv(n, b) * sp)), 256, TT_SMEM, s>>>(
-            kind, b, n, W, ldw, Z, ldz, T, sp, c->dflag.as<int>()); ::rbf::note_launch(); }
-        RBF_CUDA(cudaGetLastError());
+        RBF_CUDA(launch_early(early, k_trtri_tc, dim3(cdiv(h, 128), cdiv(h, 128), (unsigned)(cdiv(n, b) * sp)), 256,
+                              TT_SMEM, s, kind, b, n, W, ldw, Z, ldz, T, sp, c->dflag.as<int>()));
       }
       continue;
     }
@@ -525,13 +529,11 @@ rbf_status trtri_mixed(Ctx* c, const float* W, int64_t ldw, int64_t n, const flo
     const int split = (tiles < 2 * 152 && h >= 256) ? 2 : 1;
     dim3 grid(cdiv(h, TG), cdiv(h, TG), (unsigned)(cdiv(n, b) * split));
     for (int kind = 0; kind < 2; ++kind) {
-      { k_trtri_level<<<grid, 256, 0, s>>>(kind, b, n, W, ldw, Z, ldz, T, split); ::rbf::note_launch(); }
-      RBF_CUDA(cudaGetLastError());
+      RBF_CUDA(launch_early(early, k_trtri_level, grid, 256, 0, s, kind, b, n, W, ldw, Z, ldz, T, split));
     }
   }
   // Z^T stored row-major, so that products with Z^T read rows too
-  { k_transpose32<<<dim3(cdiv(n, 32), cdiv(n, 32)), 256, 0, s>>>(Z, n, ldz, Z + n * ldz); ::rbf::note_launch(); }
-  RBF_CUDA(cudaGetLastError());
+  RBF_CUDA(launch_early(early, k_transpose32, dim3(cdiv(n, 32), cdiv(n, 32)), 256, 0, s, (const float*)Z, n, ldz, Z + n * ldz));
   return RBF_OK;
 }
 
@@ -543,9 +545,9 @@ rbf_status inv_solve(Ctx* c, const float* Z, int64_t ldz, int64_t n, float* F, i
   StageTimer st(c, RBF_STAGE_INVAPPLY, s, 2.0 * (double)n * n * m);
   const float* Zt = Z + n * ldz;
   if (m <= GEMV_M) {
-    { k_inv_gemv<false><<<cdiv(n * 32, 256), 256, 0, s>>>(n, (int)m, Z, ldz, F, Y); ::rbf::note_launch(); }
+    { k_inv_gemv<false><<<cdiv(n * 32, 256), 256, 0, s>>>(n, (int)m, Z, ldz, F, Y, nullptr); ::rbf::note_launch(); }
     RBF_CUDA(cudaGetLastError());
-    { k_inv_gemv<true><<<cdiv(n * 32, 256), 256, 0, s>>>(n, (int)m, Zt, ldz, Y, F); ::rbf::note_launch(); }
+    { k_inv_gemv<true><<<cdiv(n * 32, 256), 256, 0, s>>>(n, (int)m, Zt, ldz, Y, F, nullptr); ::rbf::note_launch(); }
     RBF_CUDA(cudaGetLastError());
     return RBF_OK;
   }
@@ -572,6 +574,7 @@ rbf_status inv_solve(Ctx* c, const float* Z, int64_t ldz, int64_t n, float* F, i
 // would convert it once per row, on GB300's narrow float64 pipe), and the
 // float64 accumulation happens in the second matrix-vector launch.
 __global__ void k_round_f32(const double* __restrict__ R, int64_t cnt, float* __restrict__ F) {
+  after_previous();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < cnt) F[i] = (float)R[i];
 }
@@ -586,12 +589,11 @@ rbf_status inv_solve_acc(Ctx* c, const float* Z, int64_t ldz, int64_t n, const d
   float* F = Y + n * m;
   StageTimer st(c, RBF_STAGE_INVAPPLY, s, 2.0 * (double)n * n * m);
   const float* Zt = Z + n * ldz;
-  { k_round_f32<<<cdiv(n * m, 256), 256, 0, s>>>(R, n * m, F); ::rbf::note_launch(); }
-  RBF_CUDA(cudaGetLastError());
-  { k_inv_gemv<false><<<cdiv(n * 32, 256), 256, 0, s>>>(n, (int)m, Z, ldz, F, Y); ::rbf::note_launch(); }
-  RBF_CUDA(cudaGetLastError());
-  { k_inv_gemv<true><<<cdiv(n * 32, 256), 256, 0, s>>>(n, (int)m, Zt, ldz, Y, nullptr, X); ::rbf::note_launch(); }
-  RBF_CUDA(cudaGetLastError());
+  const bool early = not_capturing(s);
+  const unsigned g = cdiv(n * 32, 256);
+  RBF_CUDA(launch_early(early, k_round_f32, cdiv(n * m, 256), 256, 0, s, R, n * m, F));
+  RBF_CUDA(launch_early(early, k_inv_gemv<false>, g, 256, 0, s, n, (int)m, Z, ldz, (const float*)F, Y, (double*)nullptr));
+  RBF_CUDA(launch_early(early, k_inv_gemv<true>, g, 256, 0, s, n, (int)m, Zt, ldz, (const float*)Y, (float*)nullptr, X));
   return RBF_OK;
 }
 
@@ -608,7 +610,7 @@ rbf_status inv_solve_unit(Ctx* c, const float* Z, int64_t ldz, int64_t n, const 
   { k_gather_cols<<<cdiv(n * m, 256), 256, 0, s>>>(Z, n, ldz, pos, m, Y); ::rbf::note_launch(); }
   RBF_CUDA(cudaGetLastError());
   if (m <= GEMV_M) {
-    { k_inv_gemv<true><<<cdiv(n * 32, 256), 256, 0, s>>>(n, (int)m, Zt, ldz, Y, F); ::rbf::note_launch(); }
+    { k_inv_gemv<true><<<cdiv(n * 32, 256), 256, 0, s>>>(n, (int)m, Zt, ldz, Y, F, nullptr); ::rbf::note_launch(); }
     RBF_CUDA(cudaGetLastError());
     return RBF_OK;
   }
