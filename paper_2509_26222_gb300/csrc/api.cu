@@ -161,7 +161,10 @@ __global__ void k_scan_total(const Tin* in, Tout* out, int64_t n) {
 // 1024 x 8 elements in turn, each scanned in the block and offset by the
 // running total of the chunks before it; out[n] = the total.
 constexpr int SCAN1_THREADS = 1024;
-constexpr int64_t SCAN1_MAX = 32 * SCAN1_THREADS * SCAN_PER_THREAD;
+// A chunk takes 5.6 us in its turn; the tiled scan's four launches take about 14
+// for any length up to here, so three chunks is where the lines cross (65,536
+// elements: 45 us in one CTA, four kernels of 1 to 3 us tiled).
+constexpr int64_t SCAN1_MAX = 3 * SCAN1_THREADS * SCAN_PER_THREAD;
 template <class Tin, class Tout>
 __global__ void __launch_bounds__(SCAN1_THREADS) k_scan_one(const Tin* __restrict__ in, Tout* __restrict__ out,
                                                              int64_t n) {
