@@ -187,13 +187,16 @@ __global__ void __launch_bounds__(256) k_trtri_level(int kind, int64_t b, int64_
 // instructions of 128 x 128 x 16 and the split of 2 x 8,192 floats; two CTAs on
 // an SM overlap the two.  B comes as rows of K, so a thread splits two
 // neighbouring rows and stores pairs, which makes B K-major.
-// Whole inverse: a = 3,750: 893 -> 459 us; a = 2,500: 513 -> 298; a = 1,807:
+// A tile leaves by bulk operations of whole rows: with a row per lane, scattered
+// adds and stores were about a tenth of a level (four frames on the stairs
+// 12.58 -> 12.29 ms in all).  Before that, whole inverse: a = 3,750: 893 -> 459 us; a = 2,500: 513 -> 298; a = 1,807:
 // 176 -> 146.  At half-size 512 (a = 1,807 and 3,750) this kernel takes 48 and
 // 52 us for the two products, the float32 tiles 41 and 58: the line is at 1024.
 constexpr int TT_MIN = 1024;
 constexpr int TT_K = 64;
 constexpr int TT_SLICE = 128 * TT_K * 2;             // bytes of a 128 x 64 bf16 slice
 constexpr int TT_SMEM = 6 * TT_SLICE + 1024;
+constexpr int TT_ROW = 128 * 4 + 16;                 // bytes of a staged output row (padded over the banks)
 
 // x and y as three bfloat16 each (24 bits, every slice rounded to nearest), slice
 // t of x in the low and of y in the high half of q[t].  The rounding is an integer
@@ -344,28 +347,34 @@ __global__ void __launch_bounds__(256, 2) k_trtri_tc(int kind, int64_t b, int64_
     if (k0 + TT_K < ke) fetch(k0 + TT_K);
   }
   if (ok) wait();
-  // epilogue: warp w reads TMEM lanes 32 (w % 4) .., columns 64 (w / 4) .. + 63
+  // epilogue: warp w reads TMEM lanes 32 (w % 4) .., columns 64 (w / 4) .. + 63, puts
+  // them where the operands were (they are read), and a thread a row sends it off in
+  // one bulk store, or one bulk reduction where two CTAs share a tile
   if (ok) {
-    const int64_t row = i0 + 32 * (warp & 3) + lane;
     const float alpha = kind == 0 ? 1.f : -1.f;
+    const int lr = 32 * (warp & 3) + lane;
 #pragma unroll 1
     for (int cb = 0; cb < 2; ++cb) {
       const int col = 64 * (warp >> 2) + 32 * cb;
       float v[32];
       tc::tmem_ld32(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)col, v);
-      if (row < h2) {
-        float* cr = C + row * ldz + j0 + col;
-        if (split == 2) {
+      float* sr = reinterpret_cast<float*>(sm + lr * TT_ROW) + col;
 #pragma unroll
-          for (int e = 0; e < 32; ++e) atomicAdd(cr + e, alpha * v[e]);
-        } else {
-#pragma unroll
-          for (int e = 0; e < 32; e += 4)
-            *reinterpret_cast<float4*>(cr + e) =
-                make_float4(alpha * v[e], alpha * v[e + 1], alpha * v[e + 2], alpha * v[e + 3]);
-        }
-      }
+      for (int e = 0; e < 32; e += 4)
+        *reinterpret_cast<float4*>(sr + e) = make_float4(alpha * v[e], alpha * v[e + 1], alpha * v[e + 2], alpha * v[e + 3]);
     }
+    tc::fence_proxy_async();
+    __syncthreads();
+    if (tid < 128 && i0 + tid < h2) {
+      float* cr = C + (i0 + tid) * ldz + j0;
+      const uint32_t src = tc::smem_u32(sm + tid * TT_ROW);
+      if (split == 2)
+        asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], 512;" ::"l"(cr), "r"(src)
+                     : "memory");
+      else
+        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], 512;" ::"l"(cr), "r"(src) : "memory");
+    }
+    asm volatile("cp.async.bulk.commit_group;\n\tcp.async.bulk.wait_group 0;" ::: "memory");
   }
   tc::fence_before();
   __syncthreads();
