@@ -216,9 +216,9 @@ __global__ void __launch_bounds__(SCAN1_THREADS) k_scan_one(const Tin* __restric
   if (threadIdx.x == 0) out[n] = carry_s;
 }
 
+// ws: SCAN_WS buffers for the sums and offsets of the tiles, level by level
 template <class Tin, class Tout>
-static rbf_status scan_impl(Ctx* c, const Tin* in, Tout* out, int64_t n, cudaStream_t s,
-                            int slot) {
+static rbf_status scan_impl(Buf* ws, const Tin* in, Tout* out, int64_t n, cudaStream_t s) {
   if (n <= 0) {
     { k_scan_total<Tin, Tout><<<1, 1, 0, s>>>(in, out, 0); ::rbf::note_launch(); }
     RBF_CUDA(cudaGetLastError());
@@ -230,14 +230,14 @@ static rbf_status scan_impl(Ctx* c, const Tin* in, Tout* out, int64_t n, cudaStr
     return RBF_OK;
   }
   int64_t tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
-  Buf& sums = c->scratch(slot);
+  Buf& sums = ws[0];
   RBF_TRY(sums.ensure((size_t)(tiles + 1) * sizeof(Tout)));
   { k_scan_tiles<Tin, Tout><<<(unsigned)tiles, SCAN_THREADS, 0, s>>>(in, out, n, sums.as<Tout>()); ::rbf::note_launch(); }
   RBF_CUDA(cudaGetLastError());
   if (tiles > 1) {
-    Buf& offs = c->scratch(slot + 1);
+    Buf& offs = ws[1];
     RBF_TRY(offs.ensure((size_t)(tiles + 1) * sizeof(Tout)));
-    RBF_TRY((scan_impl<Tout, Tout>(c, sums.as<Tout>(), offs.as<Tout>(), tiles, s, slot + 2)));
+    RBF_TRY((scan_impl<Tout, Tout>(ws + 2, sums.as<Tout>(), offs.as<Tout>(), tiles, s)));
     { k_scan_add<Tout><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(out, n, offs.as<Tout>()); ::rbf::note_launch(); }
     RBF_CUDA(cudaGetLastError());
   }
@@ -248,12 +248,25 @@ static rbf_status scan_impl(Ctx* c, const Tin* in, Tout* out, int64_t n, cudaStr
 
 rbf_status scan_i32_to_i64(Ctx* c, const int32_t* in, int64_t* out, int64_t n, cudaStream_t s,
                            int slot) {
-  return scan_impl<int32_t, int64_t>(c, in, out, n, s, slot);
+  return scan_impl<int32_t, int64_t>(&c->ws[slot], in, out, n, s);
 }
 
 rbf_status scan_i32(Ctx* c, const int32_t* in, int32_t* out, int64_t n, cudaStream_t s,
                     int slot) {
-  return scan_impl<int32_t, int32_t>(c, in, out, n, s, slot);
+  return scan_impl<int32_t, int32_t>(&c->ws[slot], in, out, n, s);
+}
+
+rbf_status scan_i32_in(Buf* ws, const int32_t* in, int32_t* out, int64_t n, cudaStream_t s) {
+  return scan_impl<int32_t, int32_t>(ws, in, out, n, s);
+}
+
+rbf_status scan_reserve_i32(Buf* ws, int64_t n) {
+  for (int64_t m = n; m > SCAN1_MAX; ws += 2) {
+    m = (m + SCAN_TILE - 1) / SCAN_TILE;
+    RBF_TRY(ws[0].ensure((size_t)(m + 1) * sizeof(int32_t)));
+    RBF_TRY(ws[1].ensure((size_t)(m + 1) * sizeof(int32_t)));
+  }
+  return RBF_OK;
 }
 
 // ---------------------------------------------------------------------------

@@ -833,12 +833,14 @@ struct BqPlan {
   int grid = 0;
   Buf dpatches, tasks, toff, tiles64, tiles32, zd, U, u, x, r, f, part, pchunk, recs, nodes, count, start, fill,
       istart, flags, counters;
+  Buf scan[SCAN_WS];  // of the two scans (the graph records these addresses too)
   cudaGraphExec_t exec = nullptr;
   bool ran_eager = false;
   void release() {
     Buf* b[] = {&dpatches, &tasks, &toff, &tiles64, &tiles32, &zd, &U, &u, &x, &r, &f, &part, &pchunk, &recs,
                 &nodes, &count, &start, &fill, &istart, &flags, &counters};
     for (Buf* p : b) p->release();
+    for (Buf& p : scan) p.release();
     if (exec) cudaGraphExecDestroy(exec);
     exec = nullptr;
   }
@@ -972,7 +974,7 @@ static rbf_status bq_enqueue(Ctx* c, BqState* S, BqPlan& L, const BqGeom& G, cud
                                                      c->dflag.as<int>()); ::rbf::note_launch(); }
       RBF_CUDA(cudaGetLastError());
     }
-    RBF_TRY(scan_i32(c, L.count.as<int32_t>(), L.start.as<int32_t>(), L.nchunks, s, 90));
+    RBF_TRY(scan_i32_in(L.scan, L.count.as<int32_t>(), L.start.as<int32_t>(), L.nchunks, s));
     if (L.npts > 0) {
       { k_bq_fill<<<bq_blocks(L.npts), 256, 0, s>>>(dP, np, L.npts, L.pchunk.as<int2>(), L.start.as<int32_t>(),
                                                     L.fill.as<int32_t>(), L.recs.as<float4>()); ::rbf::note_launch(); }
@@ -982,7 +984,7 @@ static rbf_status bq_enqueue(Ctx* c, BqState* S, BqPlan& L, const BqGeom& G, cud
     // fill counts are reused as the per-chunk item counts
     { k_bq_items<<<bq_blocks(L.nchunks), 256, 0, s>>>(L.nchunks, L.count.as<int32_t>(), L.fill.as<int32_t>()); ::rbf::note_launch(); }
     RBF_CUDA(cudaGetLastError());
-    RBF_TRY(scan_i32(c, L.fill.as<int32_t>(), L.istart.as<int32_t>(), L.nchunks, s, 93));
+    RBF_TRY(scan_i32_in(L.scan, L.fill.as<int32_t>(), L.istart.as<int32_t>(), L.nchunks, s));
     for (size_t bk = 0; bk < L.buckets.size(); ++bk) {
       if (only_bucket >= 0 && (int)bk != only_bucket) continue;
       const int pb = L.buckets[bk].first, pe = L.buckets[bk].second;
@@ -1158,6 +1160,7 @@ static rbf_status bq_plan(Ctx* c, BqState* S, const rbf_patch* patches, int32_t 
   RBF_TRY(L.start.ensure((size_t)(maxchunks + 1) * sizeof(int32_t)));
   RBF_TRY(L.fill.ensure((size_t)(maxchunks + 1) * sizeof(int32_t)));
   RBF_TRY(L.istart.ensure((size_t)(maxchunks + 1) * sizeof(int32_t)));
+  RBF_TRY(scan_reserve_i32(L.scan, maxchunks));
   RBF_TRY(L.flags.ensure((size_t)(L.ntiles + 1) * sizeof(int)));
   RBF_TRY(L.counters.ensure(64 * sizeof(int)));
   RBF_CUDA(cudaMemcpy(L.tasks.p, tasks.data(), tasks.size() * sizeof(int4), cudaMemcpyHostToDevice));

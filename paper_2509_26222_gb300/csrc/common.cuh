@@ -269,6 +269,12 @@ rbf_status scan_i32_to_i64(Ctx* c, const int32_t* in, int64_t* out, int64_t n,
 // exclusive scan of int32 -> int32 (n + 1 entries)
 rbf_status scan_i32(Ctx* c, const int32_t* in, int32_t* out, int64_t n, cudaStream_t s,
                     int scratch_slot);
+// the same with a workspace of the caller's: for a recorded graph, which keeps
+// the addresses (the context's scratch may be replaced by a later, larger call).
+// After scan_reserve_i32(ws, m) scans of up to m entries allocate nothing.
+constexpr int SCAN_WS = 4;  // n < 2^31: two levels of tiles
+rbf_status scan_i32_in(Buf* ws, const int32_t* in, int32_t* out, int64_t n, cudaStream_t s);
+rbf_status scan_reserve_i32(Buf* ws, int64_t n);
 
 rbf_status build_center_grid(Ctx* c, cudaStream_t s);
 rbf_status refresh_center_weights(Ctx* c, cudaStream_t s);
