@@ -54,6 +54,7 @@ rbf_status Buf::ensure(size_t nbytes) {
     return cuda_fail(e, "cudaMalloc", __FILE__, __LINE__);
   }
   bytes = want;
+  ++moved;
   return RBF_OK;
 }
 

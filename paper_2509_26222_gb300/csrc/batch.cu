@@ -182,9 +182,13 @@ struct BatchState {
   std::vector<cudaEvent_t> events;
   // autotuned choice per log2(M) bucket: 0 unknown, 1 FP64, 2 mixed
   int choice[32] = {0};
+  // A graph holds the addresses of the workspaces it was recorded with: it is
+  // good as long as none of them has been replaced since (moved: workspace_moves
+  // at the recording), which a larger batch does.
   struct Graph {
     std::vector<unsigned char> key;
     cudaGraphExec_t exec = nullptr;
+    uint64_t moved = 0;
   };
   std::vector<Graph> graphs;
   std::vector<std::vector<unsigned char>> seen;  // shapes run eagerly once
@@ -217,6 +221,15 @@ static PatchGeom make_geom(const rbf_config& cfg, const rbf_patch& p) {
   G.e_gscale = cfg.kernel == RBF_KERNEL_WENDLAND ? (float)(-20.0 / (cfg.rho * cfg.rho))
                                                  : (float)(-1.0 / (cfg.sigma * cfg.sigma));
   return G;
+}
+
+static uint64_t workspace_moves(const BatchState* B) {
+  uint64_t m = 0;
+  for (const Ctx* sc : B->sub) {
+    for (const Buf& b : sc->ws) m += b.moved;
+    m += (uint64_t)sc->dflag.moved + sc->sync_flags.moved + sc->df_flags.moved;
+  }
+  return m;
 }
 
 static inline unsigned nb256(int64_t n) { return (unsigned)((n + 255) / 256); }
@@ -490,8 +503,16 @@ extern "C" rbf_status rbf_batch_update_eval(rbf_ctx* cx, const rbf_patch* patche
   for (auto& v : B->seen)
     if (v == key) seen = true;
   cudaGraphExec_t exec = nullptr;
-  for (auto& g : B->graphs)
-    if (g.key == key) exec = g.exec;
+  const uint64_t moved = workspace_moves(B);
+  for (size_t k = 0; k < B->graphs.size();) {
+    if (B->graphs[k].moved != moved) {
+      cudaGraphExecDestroy(B->graphs[k].exec);
+      B->graphs.erase(B->graphs.begin() + (std::ptrdiff_t)k);
+      continue;
+    }
+    if (B->graphs[k].key == key) exec = B->graphs[k].exec;
+    ++k;
+  }
   if (exec) {
     RBF_CUDA(cudaGraphLaunch(exec, s));
     ::rbf::note_launch();
@@ -520,7 +541,7 @@ extern "C" rbf_status rbf_batch_update_eval(rbf_ctx* cx, const rbf_patch* patche
       cudaGraphExecDestroy(B->graphs.front().exec);
       B->graphs.erase(B->graphs.begin());
     }
-    B->graphs.push_back({key, exec});
+    B->graphs.push_back({key, exec, workspace_moves(B)});
     RBF_CUDA(cudaGraphLaunch(exec, s));
     ::rbf::note_launch();
   }

@@ -45,6 +45,7 @@ enum DevFlag : int {
 struct Buf {
   void* p = nullptr;
   size_t bytes = 0;
+  uint32_t moved = 0;  // times that ensure() has replaced the allocation
   template <class T>
   T* as() const { return reinterpret_cast<T*>(p); }
   rbf_status ensure(size_t nbytes);

@@ -28,7 +28,8 @@ def batch(N, patches, M, nx, n, seed):
 
 # mixed: one-column patches have 2,048 or 4,096 chunks each (edges of 8 or 4 nodes), so that the first
 # batch's scans are tiled (from 24,577 chunks on) and the second's tile sums outgrow 64 words (131,072)
-@pytest.mark.parametrize("prec,small,large", [(1, (13, 16384, 1, 40), (64, 16384, 1, 40))])
+@pytest.mark.parametrize("prec,small,large", [(1, (13, 16384, 1, 40), (64, 16384, 1, 40)),
+                                              (0, (9, 130, 10, 400), (9, 1100, 25, 3000))])
 def test_graph_outlives_larger_batch(prec, small, large):
     from paper_2509_26222_gb300 import native as N
     N.load(build_if_missing=True)
