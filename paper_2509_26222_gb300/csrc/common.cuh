@@ -128,7 +128,7 @@ struct Ctx {
   cudaEvent_t bev[4] = {};           // fork and joins of the block stage
   bool la_ok = true;                 // look-ahead factorization allowed
   bool df_ok = true;                 // one-launch dataflow factorization allowed
-  int8_t fchoice[64] = {};           // per size bucket of 256: 0 untimed, 1 launch chain, 2 dataflow
+  int8_t fchoice[8][64] = {};        // banded blocks, per kind of band and size bucket of 256: 0 untimed, 1 launch chain, 2 dataflow
   Buf df_flags;                      // its per-tile ready flags and abort word
   uint32_t df_epoch = 0;
   cudaStream_t la_stream = nullptr;  // side stream of the look-ahead factorization

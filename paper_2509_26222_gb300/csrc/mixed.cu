@@ -634,12 +634,27 @@ static rbf_status to_f32_ends(const double* H, int64_t ldh, int64_t n, float* W,
   return RBF_OK;
 }
 
+// A dense block takes the dataflow launch below this size and the chain from it
+// on: whole update 866 / 885 us at a = 1,122 (dataflow / chain), 1,230 / 1,262 at
+// 1,806, 1,757 / 1,785 at 2,652, 2.25 / 2.20 ms at 3,025, 4.1 / 2.8 at 3,721,
+// 25.1 / 7.5 at 7,744.  The chain's trailing updates run on the tensor cores.
+constexpr int64_t DF_DENSE_MAX = 3072;
+
+// Kind of a band, for the choice below: from one end (c) or both (4 + c), c the
+// class of the half-bandwidth in 64-wide blocks (up to 2, 4, 8, more).
+static int band_kind(int64_t bw, bool two) {
+  int c = 0;
+  for (int64_t b = (bw + MB - 1) / MB; b > 2 && c < 3; b = (b + 1) / 2) ++c;
+  return (two ? 4 : 0) + c;
+}
+
 // Float32 factor of H (with the diagonal-block inverses Zd) by the dataflow
-// launch or by the launch chain.  Which is faster depends on the size (the
-// chain's tensor-core trailing updates win for large blocks): the first
-// factorization of each size bucket of 256 runs both, timed, and the bucket
-// keeps the faster.  Stream capture, batched sub-contexts and blocks beyond
-// DF_NMAX use the chain.  The dataflow launch eliminates a band from both ends
+// launch or by the launch chain.  Which is faster depends on the size and the
+// band: dense blocks go by DF_DENSE_MAX; the first banded factorization of each
+// kind of band and size bucket of 256 runs both, timed, and keeps the faster.
+// (Kept by the size alone, a dense block took the choice of the banded one
+// before it, which the dataflow launch mostly wins.)  Stream capture, batched
+// sub-contexts and blocks beyond DF_NMAX use the chain.  The dataflow launch eliminates a band from both ends
 // (*ends) where the caller can use that factor, nothing reads all of its
 // triangle, and the ends are at least twice the band apart, so that most of the
 // two chains run side by side.
@@ -664,13 +679,14 @@ rbf_status potrf_mixed(Ctx* c, const double* H, int64_t ldh, int64_t n, float* W
   RBF_CUDA(cudaStreamIsCapturing(s, &cap0));
   if (!(c->la_ok && c->df_ok && n <= DF_NMAX && cap0 == cudaStreamCaptureStatusNone)) return chain();
   const int b = (int)(n / 256);
-  int8_t& pick = c->fchoice[b < 64 ? b : 63];
+  int8_t dense = n < DF_DENSE_MAX ? 2 : 1;
+  int8_t& pick = bw < n ? c->fchoice[band_kind(bw, two)][b < 64 ? b : 63] : dense;
   if (pick == 1) return chain();
   if (pick == 2) {
     const rbf_status st = dataflow();
     return st != RBF_ERANGE ? st : chain();
   }
-  // first block of this size: time both (the dataflow result is kept)
+  // first banded block of this kind and size: time both (the dataflow result is kept)
   cudaEvent_t ev[3];
   for (auto& e : ev) RBF_CUDA(cudaEventCreate(&e));
   RBF_CUDA(cudaEventRecord(ev[0], s));
