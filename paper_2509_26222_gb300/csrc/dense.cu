@@ -17,7 +17,10 @@
 //    timeout sets a status bit) before consuming a solved block.
 #include <math.h>
 
+#include <type_traits>
+
 #include "common.cuh"
+#include "recip.cuh"
 
 namespace rbf {
 
@@ -25,16 +28,6 @@ constexpr int NB = 32;   // block of the triangular solves
 constexpr int PB = 16;   // block column of the factorization
 constexpr int UT = 32;   // tile of the trailing update
 constexpr int PT = 256;  // threads of a factorization CTA
-
-// 1 / d for a positive normal d: the hardware's approximation (about 20 bits)
-// and one third-order step y (1 + e + e^2), e = 1 - d y (Householder's method
-// for the reciprocal), whose error e^3 lies below float64 rounding.
-__device__ __forceinline__ double rcp_pos(double d) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-  const double e = fma(-d, y, 1.0);
-  return fma(y, fma(e, e, e), y);
-}
 
 // ---------------------------------------------------------------------------
 // Step k of the factorization, one CTA per SM.
@@ -79,7 +72,7 @@ __global__ void __launch_bounds__(PT) k_potrf_step(PotrfStep P) {
   __shared__ double Lk[PB][PB + 1];  // L[k block, k - 1]
   __shared__ double rs[PB];          // D^-1/2
   __shared__ double Pi[2][PB][UT + 1], Pj[2][PB][UT + 1];
-  __shared__ int nxt[2];
+  __shared__ int nxt[2], redo;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   after_previous();
   double* __restrict__ A = P.A;
@@ -106,13 +99,16 @@ __global__ void __launch_bounds__(PT) k_potrf_step(PotrfStep P) {
     }
     D[i][j] = dv;
     __syncthreads();
-    if (warp == 0) {
+    // in: D; out: D = V, U = V D^-1, rs.  Warp 0; true if a pivot lies outside the
+    // range of rcp_pos (nothing of the result is used then, unless ANY).
+    auto eliminate = [&](auto any) {
+      constexpr bool ANY = decltype(any)::value;
       const int ri = lane & 15, h = lane >> 4;
       double a[PB / 2];
 #pragma unroll
       for (int c = 0; c < PB / 2; ++c) a[c] = D[ri][2 * c + h];
       __syncwarp();
-      bool bad = false;
+      bool bad = false, odd = false;
 #pragma unroll
       for (int t = 0; t < PB; ++t) {
         const double v = __shfl_sync(0xffffffffu, a[t >> 1], ri + 16 * (t & 1));  // column t of row ri
@@ -121,7 +117,8 @@ __global__ void __launch_bounds__(PT) k_potrf_step(PotrfStep P) {
           bad = true;
           d = 1.0;
         }
-        const double u = v * rcp_pos(d);
+        odd |= !rcp_pos_range(d);
+        const double u = ANY ? v / d : v * rcp_pos(d);
         if (h == 0) {
           D[ri][t] = ri == t ? d : v;
           U[ri][t] = u;
@@ -132,9 +129,14 @@ __global__ void __launch_bounds__(PT) k_potrf_step(PotrfStep P) {
           if (2 * c + h > t) a[c] = fma(-u, vk, a[c]);
         }
       }
-      if (bad && lane == 0 && blockIdx.x == 0) atomicOr(P.flag, DEV_NOT_SPD);
+      if (bad && (ANY || !odd) && lane == 0 && blockIdx.x == 0) atomicOr(P.flag, DEV_NOT_SPD);
       __syncwarp();
       if (h == 0) rs[ri] = rsqrt(D[ri][ri]);
+      return odd;
+    };
+    if (warp == 0) {
+      const bool odd = eliminate(std::false_type{});
+      if (lane == 0) redo = odd ? 1 : 0;
     }
     if (kp) {  // the rows' own update, beside the chain of the diagonal tile
       double acc = 0.0;
@@ -143,8 +145,15 @@ __global__ void __launch_bounds__(PT) k_potrf_step(PotrfStep P) {
       x -= acc;
     }
     __syncthreads();
+    if (redo) {  // a subnormal, huge or infinite pivot: again, with the language's division
+      D[i][j] = dv;
+      __syncthreads();
+      if (warp == 0) eliminate(std::true_type{});
+      __syncthreads();
+    }
     if (blockIdx.x == 0) {
-      const double l = i == j ? D[i][i] * rs[i] : (j < i ? D[i][j] * rs[j] : 0.0);
+      double l = j <= i ? D[i][j] * rs[j] : 0.0;  // D rsqrt(D) on the diagonal
+      if (i == j && isinf(D[i][i])) l = D[i][i];  // (an infinite ridge: its weight stays zero)
       if (P.npanel > 1) P.dt[tid] = l;
       else if (i < kb && j <= i) A[(k + i) * lda + k + j] = l;  // this CTA alone has read the tile
     }
