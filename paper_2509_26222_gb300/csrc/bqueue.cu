@@ -173,13 +173,14 @@ __device__ __forceinline__ void bq_add_split(unsigned* G2, unsigned long long v)
   if (h) atomicAdd(G2 + 1, h);
 }
 
-// m z in 2^-64 units, exactly (m = q 2^-52, q < 2^53), added to a 128-bit sum
-__device__ __forceinline__ void bq_add_mz(unsigned long long* u2, unsigned long long q, float z) {
+// m z in 2^-64 units, the exact product truncated to a whole number of them
+// (m = q 2^-k, q < 2^63), added to a 128-bit sum
+__device__ __forceinline__ void bq_add_mz(unsigned long long* u2, unsigned long long q, int k, float z) {
   const unsigned bits = __float_as_uint(z);
   const int ex = (bits >> 23) & 255;
   const unsigned long long mant = (bits & 0x7fffffu) | (ex ? 0x800000u : 0u);
   unsigned long long lo = q * mant, hi = __umul64hi(q, mant);
-  const int sh = (ex ? ex : 1) - 138;  // z = mant 2^(ex - 150)
+  const int sh = (ex ? ex : 1) - 86 - k;  // z = mant 2^(ex - 150)
   if (sh >= 0) {
     if (sh >= 64) {
       hi = sh < 128 ? lo << (sh - 64) : 0ull;
@@ -204,9 +205,42 @@ __device__ __forceinline__ void bq_add_mz(unsigned long long* u2, unsigned long 
   u2[1] += hi + ((o + lo < o) ? 1ull : 0ull);
 }
 
+// The value of such a sum.  A negative one is negated first: its low word, close to
+// 2^64 for a sum close to zero, would lose all but 2^-54 of it.
+__device__ __forceinline__ double bq_sum_value(unsigned long long lo, unsigned long long hi) {
+  const bool neg = (long long)hi < 0;
+  if (neg) {
+    lo = ~lo + 1ull;
+    hi = ~hi + (lo == 0ull ? 1ull : 0ull);
+  }
+  const double v = (double)hi + ldexp((double)lo, -64);
+  return neg ? -v : v;
+}
+
+// m > 0 as q 2^-k with all its bits (k such that q has 63 or 53 of them), and
+// rounded to 2^-52
+struct BqM {
+  unsigned long long q, q52;
+  int k;
+};
+__device__ __forceinline__ BqM bq_fixed(FF m) {
+  const int k = min(189 - (int)(__float_as_uint(m.hi) >> 23), 122);  // hi 2^k in [2^62, 2^63) from hi = 2^-60 on
+  const float f = __int_as_float((k + 127) << 23);
+  BqM r;
+  r.k = k;
+  r.q = __float2ull_rn(m.hi * f) + (unsigned long long)__float2ll_rn(m.lo * f);
+  r.q52 = k < 116 ? ((r.q >> (k - 53)) + 1ull) >> 1 : 0ull;
+  return r;
+}
+__device__ __forceinline__ BqM bq_fixed(double m) {
+  const unsigned long long bits = (unsigned long long)__double_as_longlong(m);
+  const int ex = (int)(bits >> 52);
+  return {(bits & 0xfffffffffffffull) | (ex ? 1ull << 52 : 0ull), __double2ull_rn(ldexp(m, 52)), 1075 - (ex ? ex : 1)};
+}
+
 // A warp a point.  What bounds it is instruction issue: every float64 instruction
 // costs 19 cycles of the SM, so none is left on the Wendland path (the cell comes
-// with the record, m as 52-bit fixed point from float-float, m z in integers),
+// with the record, m as fixed point from float-float, m z in integers),
 // the in-support nodes are compacted before m is formed, and rows r and
 // K - 1 - r of the pair triangle share a pass of K + 1 lanes.
 // 256 patches, 2.8 M points: 8.6 -> 4.4 ms.
@@ -275,30 +309,33 @@ __global__ void __launch_bounds__(256) k_bq_gram(const BqPatch* __restrict__ P, 
         K += __popc(mask);
       }
       __syncwarp();
-      // m (2^52 units per 1) of the nodes in support, and m z into this warp's
+      // m (for the products in 2^52 units per 1) of the nodes in support, and m z into this warp's
       // private 128-bit sums (2^64 units per 1): the lanes hold distinct nodes,
       // and the warp's points come one at a time
       for (int t = lane; t < K; t += 32) {
         const int wi = sid[wid][t] & 255, wj = sid[wid][t] >> 8, li = wj * W + wi;
         const FF cx = nodex[wi], cy = nodey[wj];
-        unsigned long long mq;
+        BqM m;
         if (G.kernel == RBF_KERNEL_WENDLAND) {
           // m = (1 - s)^4 (4 s + 1), s = |p - c| / rho, in float-float
-          const FF dx = ff_two_sum(__fsub_rn(px, cx.hi), -cx.lo);  // px - cx.hi is exact
+          // (px - cx.hi is exact for operands within a factor of two of each other;
+          // for others, near a coordinate of zero, it is rounded, which leaves d about
+          // 24 bits and moves the weights by up to 1e-7)
+          const FF dx = ff_two_sum(__fsub_rn(px, cx.hi), -cx.lo);
           const FF dy = ff_two_sum(__fsub_rn(py, cy.hi), -cy.lo);
           const FF sr = ff_mul(ff_sqrt(ff_add(ff_mul(dx, dx), ff_mul(dy, dy))), inv_rho);
           const FF t1 = ff_add({1.f, 0.f}, {-sr.hi, -sr.lo});
           const FF t2 = ff_mul(t1, t1);
           const FF mm = ff_mul(ff_mul(t2, t2), ff_add({4.f * sr.hi, 4.f * sr.lo}, {1.f, 0.f}));
-          mq = __float2ull_rn(ldexpf(mm.hi, 52)) + (unsigned long long)__float2ll_rn(ldexpf(mm.lo, 52));
+          m = bq_fixed(mm);
         } else {
           const double ex = (double)px - ((double)cx.hi + (double)cx.lo);
           const double ey = (double)py - ((double)cy.hi + (double)cy.lo);
-          mq = __double2ull_rn(ldexp(row_value(G.kernel, ex * ex + ey * ey, G.inv_rho, G.g_scale, G.g_inv2s2), 52));
+          m = bq_fixed(row_value(G.kernel, ex * ex + ey * ey, G.inv_rho, G.g_scale, G.g_inv2s2));
         }
         sid[wid][t] = li;
-        smq[wid][t] = mq;
-        bq_add_mz(sU + 2 * li, mq, pz);
+        smq[wid][t] = m.q52;
+        bq_add_mz(sU + 2 * li, m.q, m.k, pz);
       }
       __syncwarp();
       // products m_a m_b in integer arithmetic: the exact 106-bit product of
@@ -390,7 +427,7 @@ __global__ void __launch_bounds__(256) k_bq_merge(const BqPatch* __restrict__ P,
   if (i == l && threadIdx.x < 64) {
     const int r = threadIdx.x;
     const long long v = B.vec0 + (long long)i * 64 + r;
-    u[v] = r < ri ? (double)(long long)Ut[2 * v + 1] + ldexp((double)Ut[2 * v], -64) : 0.0;
+    u[v] = r < ri ? bq_sum_value(Ut[2 * v], Ut[2 * v + 1]) : 0.0;
   }
 }
 
