@@ -306,21 +306,35 @@ inline cudaError_t cooperative_launch(const void* f, dim3 g, dim3 b, void** args
 // for kernels that call after_previous() before they touch global memory.  The
 // call also lets the next such launch be placed.  early = false (stream capture,
 // single launches): an ordinary launch.
+// cz: blocks of a cluster along z (1: no clusters).
 template <class... P, class... A>
-inline cudaError_t launch_early(bool early, void (*f)(P...), dim3 g, dim3 b, size_t smem, cudaStream_t s, A&&... args) {
+inline cudaError_t launch_early_z(bool early, unsigned cz, void (*f)(P...), dim3 g, dim3 b, size_t smem, cudaStream_t s,
+                                  A&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = g;
   cfg.blockDim = b;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute at;
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = early ? 1 : 0;
+  cudaLaunchAttribute at[2];
+  unsigned na = 0;
+  if (early) {
+    at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[na++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cz > 1) {
+    at[na].id = cudaLaunchAttributeClusterDimension;
+    at[na].val.clusterDim.x = at[na].val.clusterDim.y = 1;
+    at[na++].val.clusterDim.z = cz;
+  }
+  cfg.attrs = at;
+  cfg.numAttrs = na;
   cudaError_t e = cudaLaunchKernelEx(&cfg, f, std::forward<A>(args)...);
   if (e == cudaSuccess) note_launch();
   return e;
+}
+template <class... P, class... A>
+inline cudaError_t launch_early(bool early, void (*f)(P...), dim3 g, dim3 b, size_t smem, cudaStream_t s, A&&... args) {
+  return launch_early_z(early, 1u, f, g, b, smem, s, std::forward<A>(args)...);
 }
 __device__ __forceinline__ void after_previous() {
   asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");

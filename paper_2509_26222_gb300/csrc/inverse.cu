@@ -20,6 +20,7 @@
 
 #include "common.cuh"
 #include "tc_util.cuh"
+#include "tiles.cuh"
 
 namespace rbf {
 namespace {
@@ -177,25 +178,35 @@ __global__ void __launch_bounds__(256) k_trtri_level(int kind, int64_t b, int64_
 }
 
 // The same products for the levels whose half has TT_MIN rows or more, on the
-// tensor cores: one 128 x 128 tile of the output per CTA (or half of its K
-// range), C = A B with float32 operands split into three bfloat16 slices on
-// their way into shared memory and the six slice products down to 2^-24 of
-// |A| |B| accumulated in float32 in tensor memory, as in the trailing update.
+// tensor cores: one 128 x 128 tile of the output per CTA, C = A B with float32
+// operands split into three bfloat16 slices (h, m, l) on their way into shared
+// memory and their products accumulated in float32 in tensor memory.
 //
-// The large levels are nearly all of the n^3 / 3 multiply-adds.  On the float32 pipe 64 x 64 tiles reach 16 to 20 TFLOP/s there,
-// bound by their shared-memory loads.  Here a chunk of K = 64 costs a CTA 24
-// instructions of 128 x 128 x 16 and the split of 2 x 8,192 floats; two CTAs on
-// an SM overlap the two.  B comes as rows of K, so a thread splits two
-// neighbouring rows and stores pairs, which makes B K-major.
-// A tile leaves by bulk operations of whole rows: with a row per lane, scattered
-// adds and stores were about a tenth of a level (four frames on the stairs
-// 12.58 -> 12.29 ms in all).  Before that, whole inverse: a = 3,750: 893 -> 459 us; a = 2,500: 513 -> 298; a = 1,807:
-// 176 -> 146.  At half-size 512 (a = 1,807 and 3,750) this kernel takes 48 and
-// 52 us for the two products, the float32 tiles 41 and 58: the line is at 1024.
+// The large levels are nearly all of the n^3 / 3 multiply-adds.  On the float32
+// pipe 64 x 64 tiles reach 16 to 20 TFLOP/s there, bound by their shared-memory
+// loads.  Here a chunk of K = 64 costs a CTA 24 or 32 instructions of
+// 128 x 128 x 16 and the split of 2 x 8,192 floats; two CTAs on an SM overlap the
+// two.  B comes as rows of K, so a thread splits two neighbouring rows and stores
+// pairs, which makes B K-major.  At half-size 512 this kernel takes as long as the
+// float32 tiles (48 + 52 us and 41 + 58 for the two products): the line is at 1024.
+// Whole inverse, float32 tiles and now: n = 1,810 225 / 170 us, 2,500 517 / 279,
+// 3,750 936 / 466, 5,000 1,959 / 1,000.
+//
+// No further from 64 bits than float32 multiply-adds (0.77 to 1.00 times, block by
+// block), because
+//  * the product h h and the small ones have an accumulator each: added to one,
+//    every small product was rounded to the sum of the large ones (2.1 to 2.4);
+//  * where a level has fewer tiles than two per SM and two CTAs take half of K
+//    each, they are a cluster and swap halves of their accumulators, which are
+//    added before the one rounding (rounded apart and added in memory: up to 1.03);
+//  * the first product, whose errors the second one amplifies, takes all products
+//    but l l, the second one h h, h m, h l and m m (six for both: up to 1.0004).
+// The three cost 6 to 10 % of the inverse.
 constexpr int TT_MIN = 1024;
 constexpr int TT_K = 64;
 constexpr int TT_SLICE = 128 * TT_K * 2;             // bytes of a 128 x 64 bf16 slice
 constexpr int TT_SMEM = 6 * TT_SLICE + 1024;
+constexpr uint32_t TT_COLS = 256;
 constexpr int TT_ROW = 128 * 4 + 16;                 // bytes of a staged output row (padded over the banks)
 
 // x and y as three bfloat16 each (24 bits, every slice rounded to nearest), slice
@@ -234,14 +245,14 @@ __global__ void __launch_bounds__(256, 2) k_trtri_tc(int kind, int64_t b, int64_
     if (blockIdx.z & 1) kb = mid;
     else ke = mid;
   }
-  if (kb >= ke) return;
+  const bool some = kb < ke;  // (the second half of a short K may be empty)
   const float* A = kind == 0 ? W + r2 * ldw + r1 : Z + r2 * ldz + r2;
   const int64_t lda = kind == 0 ? ldw : ldz;
   const float* B = kind == 0 ? Z + r1 * ldz + r1 : T + r2 * ldz + r1;
   float* C = (kind == 0 ? T : Z) + r2 * ldz + r1;
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(tt_raw) + 1023) & ~(uintptr_t)1023);
   after_previous();
-  if (warp == 0) tc::tmem_alloc(&tmem_slot, 128);
+  if (warp == 0) tc::tmem_alloc(&tmem_slot, TT_COLS);
   if (tid == 0) tc::mbar_init(&mbar, 1);
   tc::fence_before();
   __syncthreads();
@@ -298,7 +309,7 @@ __global__ void __launch_bounds__(256, 2) k_trtri_tc(int kind, int64_t b, int64_
     ok = ok_s != 0;
     phase ^= 1;
   };
-  fetch(kb);
+  if (some) fetch(kb);
   for (int64_t k0 = kb; k0 < ke && ok; k0 += TT_K) {
     if (k0 > kb) wait();
     if (!ok) break;
@@ -333,52 +344,87 @@ __global__ void __launch_bounds__(256, 2) k_trtri_tc(int kind, int64_t b, int64_
     __syncthreads();
     tc::fence_after();
     if (tid == 0) {
-      const int pa[6] = {0, 0, 1, 0, 1, 2}, pb[6] = {0, 1, 0, 2, 1, 0};
+      const int pa[8] = {0, 0, 1, 0, 1, 2, 1, 2}, pb[8] = {0, 1, 0, 2, 1, 0, 2, 1};
 #pragma unroll
-      for (int q = 0; q < 6; ++q) {
+      for (int q = 0; q < 8; ++q) {
+        if (q >= 6 && kind != 0) break;
         const uint64_t ad = tc::sdesc_sw128(tc::smem_u32(sm + pa[q] * TT_SLICE));
         const uint64_t bd = tc::sdesc_sw128(tc::smem_u32(sm + (3 + pb[q]) * TT_SLICE));
 #pragma unroll
         for (int kk = 0; kk < TT_K / 16; ++kk)
-          tc::mma_bf16(tmem, ad + (uint64_t)(2 * kk), bd + (uint64_t)(2 * kk), (k0 > kb || q > 0 || kk > 0) ? 1u : 0u);
+          tc::mma_bf16(tmem + (q ? 128u : 0u), ad + (uint64_t)(2 * kk), bd + (uint64_t)(2 * kk),
+                       (k0 > kb || q > 1 || kk > 0) ? 1u : 0u);
       }
       tc::mma_commit(&mbar);
     }
     if (k0 + TT_K < ke) fetch(k0 + TT_K);
   }
-  if (ok) wait();
-  // epilogue: warp w reads TMEM lanes 32 (w % 4) .., columns 64 (w / 4) .. + 63, puts
-  // them where the operands were (they are read), and a thread a row sends it off in
-  // one bulk store, or one bulk reduction where two CTAs share a tile
-  if (ok) {
-    const float alpha = kind == 0 ? 1.f : -1.f;
-    const int lr = 32 * (warp & 3) + lane;
+  if (ok && some) wait();
+  // epilogue: warp w reads TMEM lanes 32 (w % 4) .., puts a row a lane where the
+  // operands were (they are read), and a thread a row sends it off in one bulk store
+  const float alpha = kind == 0 ? 1.f : -1.f;
+  const int lr = 32 * (warp & 3) + lane, q = warp >> 2;
+  const uint32_t tl = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
+  float v[32], v2[32];
+  auto load = [&](int col) {
+    tc::tmem_ld32(tl + (uint32_t)col, v);
+    tc::tmem_ld32(tl + (uint32_t)(128 + col), v2);
+#pragma unroll
+    for (int e = 0; e < 32; ++e) {
+      if (!some) v[e] = v2[e] = 0.f;
+    }
+  };
+  auto send = [&](int col, int bytes) {
+    tc::fence_proxy_async();
+    __syncthreads();
+    if (tid < 128 && i0 + tid < h2)
+      asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(C + (i0 + tid) * ldz + j0 + col),
+                   "r"(tc::smem_u32(sm + tid * TT_ROW)), "r"(bytes)
+                   : "memory");
+    asm volatile("cp.async.bulk.commit_group;\n\tcp.async.bulk.wait_group 0;" ::: "memory");
+  };
+  if (split == 2) {
+    // columns 64 rank .. + 63 are this CTA's: the others' two accumulators go to the peer
+    const uint32_t rank = blockIdx.z & 1;
+    tc::cluster_arrive();
+    load(64 * (int)(rank ^ 1) + 32 * q);
+    tc::cluster_wait();  // both have read their operands
+    const uint32_t to = tc::cluster_addr(tc::smem_u32(sm + lr * TT_ROW) + 128u * q, rank ^ 1);
+#pragma unroll
+    for (int e = 0; e < 32; e += 4) {
+      tc::cluster_store4(to + 4 * e, v[e], v[e + 1], v[e + 2], v[e + 3]);
+      tc::cluster_store4(to + 256 + 4 * e, v2[e], v2[e + 1], v2[e + 2], v2[e + 3]);
+    }
+    tc::cluster_arrive();
+    load(64 * (int)rank + 32 * q);
+    tc::cluster_wait();
+    float* sr = reinterpret_cast<float*>(sm + lr * TT_ROW) + 32 * q;
+#pragma unroll
+    for (int e = 0; e < 32; e += 4) {
+      const float4 a = *reinterpret_cast<const float4*>(sr + e), c = *reinterpret_cast<const float4*>(sr + 64 + e);
+      auto sum = [&](float x, float y, int k) {
+        const FF s = ff_two_sum(v[e + k], x);
+        return alpha * (s.hi + (s.lo + (v2[e + k] + y)));
+      };
+      *reinterpret_cast<float4*>(sr + e) = make_float4(sum(a.x, c.x, 0), sum(a.y, c.y, 1), sum(a.z, c.z, 2), sum(a.w, c.w, 3));
+    }
+    if (ok) send(64 * (int)rank, 256);
+  } else if (ok) {
 #pragma unroll 1
     for (int cb = 0; cb < 2; ++cb) {
-      const int col = 64 * (warp >> 2) + 32 * cb;
-      float v[32];
-      tc::tmem_ld32(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)col, v);
+      const int col = 64 * q + 32 * cb;
+      load(col);
       float* sr = reinterpret_cast<float*>(sm + lr * TT_ROW) + col;
 #pragma unroll
       for (int e = 0; e < 32; e += 4)
-        *reinterpret_cast<float4*>(sr + e) = make_float4(alpha * v[e], alpha * v[e + 1], alpha * v[e + 2], alpha * v[e + 3]);
+        *reinterpret_cast<float4*>(sr + e) = make_float4(alpha * (v[e] + v2[e]), alpha * (v[e + 1] + v2[e + 1]),
+                                                         alpha * (v[e + 2] + v2[e + 2]), alpha * (v[e + 3] + v2[e + 3]));
     }
-    tc::fence_proxy_async();
-    __syncthreads();
-    if (tid < 128 && i0 + tid < h2) {
-      float* cr = C + (i0 + tid) * ldz + j0;
-      const uint32_t src = tc::smem_u32(sm + tid * TT_ROW);
-      if (split == 2)
-        asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], 512;" ::"l"(cr), "r"(src)
-                     : "memory");
-      else
-        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], 512;" ::"l"(cr), "r"(src) : "memory");
-    }
-    asm volatile("cp.async.bulk.commit_group;\n\tcp.async.bulk.wait_group 0;" ::: "memory");
+    send(0, 512);
   }
   tc::fence_before();
   __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tmem, 128);
+  if (warp == 0) tc::tmem_dealloc(tmem, TT_COLS);
 }
 
 // Y = Z F (forward, Z lower) or Y = Zt F (backward, Zt = Z^T upper) for
@@ -524,12 +570,12 @@ rbf_status trtri_mixed(Ctx* c, const float* W, int64_t ldw, int64_t n, const flo
         RBF_CUDA(cudaFuncSetAttribute(k_trtri_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, TT_SMEM));
         attr[c->device & 63] = true;
       }
-      // fewer tiles than two per SM: K in two halves (0 + a + b = 0 + b + a exactly)
+      // fewer tiles than two per SM: K in two halves, by a pair of CTAs
       const int64_t tt = (int64_t)cdiv(h, 128) * cdiv(h, 128) * cdiv(n, b);
       const int sp = tt < 2 * 152 ? 2 : 1;
       for (int kind = 0; kind < 2; ++kind) {
-        RBF_CUDA(launch_early(early, k_trtri_tc, dim3(cdiv(h, 128), cdiv(h, 128), (unsigned)(cdiv(n, b) * sp)), 256,
-                              TT_SMEM, s, kind, b, n, W, ldw, Z, ldz, T, sp, c->dflag.as<int>()));
+        RBF_CUDA(launch_early_z(early, (unsigned)sp, k_trtri_tc, dim3(cdiv(h, 128), cdiv(h, 128), (unsigned)(cdiv(n, b) * sp)),
+                                256, TT_SMEM, s, kind, b, n, W, ldw, Z, ldz, T, sp, c->dflag.as<int>()));
       }
       continue;
     }
