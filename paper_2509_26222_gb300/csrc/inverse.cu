@@ -210,11 +210,16 @@ constexpr uint32_t TT_COLS = 256;
 constexpr int TT_ROW = 128 * 4 + 16;                 // bytes of a staged output row (padded over the banks)
 
 // x and y as three bfloat16 each (24 bits, every slice rounded to nearest), slice
-// t of x in the low and of y in the high half of q[t].  The rounding is an integer
-// addition: the conversion instruction runs at a fraction of the rate.
+// t of x in the low and of y in the high half of q[t].  The first slice comes from
+// the conversion instruction, which keeps a NaN a NaN; the others' rounding is an
+// integer addition (which takes the GPU's NaN, 0x7fffffff, to -0), because the
+// conversion runs at a fraction of the rate.
 __device__ __forceinline__ void split3(float x, float y, uint32_t (&q)[3]) {
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(q[0]) : "f"(y), "f"(x));
+  x -= __uint_as_float(q[0] << 16);
+  y -= __uint_as_float(q[0] & 0xffff0000u);
 #pragma unroll
-  for (int t = 0; t < 3; ++t) {
+  for (int t = 1; t < 3; ++t) {
     const uint32_t a = (__float_as_uint(x) + 0x8000u) & 0xffff0000u, b = (__float_as_uint(y) + 0x8000u) & 0xffff0000u;
     q[t] = __byte_perm(a, b, 0x7632);
     x -= __uint_as_float(a);
