@@ -189,8 +189,8 @@ __global__ void __launch_bounds__(256) k_trtri_level(int kind, int64_t b, int64_
 // two.  B comes as rows of K, so a thread splits two neighbouring rows and stores
 // pairs, which makes B K-major.  At half-size 512 this kernel takes as long as the
 // float32 tiles (48 + 52 us and 41 + 58 for the two products): the line is at 1024.
-// Whole inverse, float32 tiles and now: n = 1,810 225 / 170 us, 2,500 517 / 279,
-// 3,750 936 / 466, 5,000 1,959 / 1,000.
+// Whole inverse, float32 tiles and now: n = 1,810 225 / 166 us, 2,500 517 / 269,
+// 3,750 936 / 443, 5,000 1,959 / 922.
 //
 // No further from 64 bits than float32 multiply-adds (0.77 to 1.00 times, block by
 // block), because
@@ -209,21 +209,16 @@ constexpr int TT_SMEM = 6 * TT_SLICE + 1024;
 constexpr uint32_t TT_COLS = 256;
 constexpr int TT_ROW = 128 * 4 + 16;                 // bytes of a staged output row (padded over the banks)
 
-// x and y as three bfloat16 each (24 bits, every slice rounded to nearest), slice
-// t of x in the low and of y in the high half of q[t].  The first slice comes from
-// the conversion instruction, which keeps a NaN a NaN; the others' rounding is an
-// integer addition (which takes the GPU's NaN, 0x7fffffff, to -0), because the
-// conversion runs at a fraction of the rate.
+// x and y as three bfloat16 each (24 bits, every slice rounded to nearest; a NaN
+// stays one), slice t of x in the low and of y in the high half of q[t].  (With the
+// rounding as an integer addition, inverse of 3,750 rows 474 us; with the
+// conversion instruction 443.)
 __device__ __forceinline__ void split3(float x, float y, uint32_t (&q)[3]) {
-  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(q[0]) : "f"(y), "f"(x));
-  x -= __uint_as_float(q[0] << 16);
-  y -= __uint_as_float(q[0] & 0xffff0000u);
 #pragma unroll
-  for (int t = 1; t < 3; ++t) {
-    const uint32_t a = (__float_as_uint(x) + 0x8000u) & 0xffff0000u, b = (__float_as_uint(y) + 0x8000u) & 0xffff0000u;
-    q[t] = __byte_perm(a, b, 0x7632);
-    x -= __uint_as_float(a);
-    y -= __uint_as_float(b);
+  for (int t = 0; t < 3; ++t) {
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(q[t]) : "f"(y), "f"(x));
+    x -= __uint_as_float(q[t] << 16);
+    y -= __uint_as_float(q[t] & 0xffff0000u);
   }
 }
 
