@@ -607,6 +607,7 @@ __device__ __forceinline__ float bq_quad_sum(float s) {
 }
 
 constexpr int BQ_NEAR = 6;  // band tiles next to the diagonal whose loads run ahead
+constexpr int BQ_FAR = 4;   // tiles farther off whose loads are in flight together (x 64 <= 256 threads)
 
 // persistent: CTAs pull patches; solve H' c = r with the float32 factor
 // (forward then backward block substitution within the band), then x += c.
@@ -615,12 +616,13 @@ constexpr int BQ_NEAR = 6;  // band tiles next to the diagonal whose loads run a
 // latency of its loads: so the tiles nearest the diagonal (a lattice of up to 63
 // columns at rho = 3 h has six) and the diagonal inverse of the next row are
 // loaded while this row is reduced, and the last solved blocks stay in shared
-// memory.  Tiles farther off follow with loads of their own.  256 patches, nb up
-// to 64: three sweeps 2.14 -> 1.98 ms.
+// memory.  Tiles farther off follow in groups.  256 patches, nb up to 64: three
+// sweeps 2.14 -> 1.98 ms.  Batch of four patches of 128 x 128 (12 tiles): 21.5 ms
+// with the far tiles one by one, 20.2 in threes, 19.5 in fours (and 36 bytes of spills).
 __global__ void __launch_bounds__(256) k_bq_solve(const BqPatch* __restrict__ P, int np, const float* __restrict__ Wt,
                                                   const float* __restrict__ Zd, const double* __restrict__ r,
                                                   float* __restrict__ f, double* __restrict__ x, int* __restrict__ counter) {
-  __shared__ float acc[64], vk[64], ring[8][64];  // block k of the solution in ring[k % 8]
+  __shared__ float acc[64], vk[BQ_FAR][64], ring[8][64];  // block k of the solution in ring[k % 8]
   __shared__ int cur;
   const int tid = threadIdx.x, row = tid >> 2, part = tid & 3;
   for (;;) {
@@ -649,12 +651,17 @@ __global__ void __launch_bounds__(256) k_bq_solve(const BqPatch* __restrict__ P,
     for (int b = 0; b < nb; ++b) {
       const float rb = part == 0 ? (float)rv[b * 64 + row] : 0.f;
       float s = 0.f;
-      for (int k = b - bwb > 0 ? b - bwb : 0; k < b - BQ_NEAR; ++k) {
-        if (tid < 64) vk[tid] = fv[k * 64 + tid];
-        float t[16];
-        bq_load16(gtile(b, k), false, t);
+      for (int k = b - bwb > 0 ? b - bwb : 0; k < b - BQ_NEAR; k += BQ_FAR) {
+        const int ng = b - BQ_NEAR - k < BQ_FAR ? b - BQ_NEAR - k : BQ_FAR;
+        if (tid < ng * 64) vk[tid >> 6][tid & 63] = fv[k * 64 + tid];
+        float t[BQ_FAR][16];
+#pragma unroll
+        for (int j = 0; j < BQ_FAR; ++j)
+          if (j < ng) bq_load16(gtile(b, k + j), false, t[j]);
         __syncthreads();
-        s += bq_dot16(t, vk);
+#pragma unroll
+        for (int j = 0; j < BQ_FAR; ++j)
+          if (j < ng) s += bq_dot16(t[j], vk[j]);
         __syncthreads();
       }
 #pragma unroll
@@ -686,12 +693,17 @@ __global__ void __launch_bounds__(256) k_bq_solve(const BqPatch* __restrict__ P,
     for (int b = nb - 1; b >= 0; --b) {
       const float yb = part == 0 ? fv[b * 64 + row] : 0.f;
       float s = 0.f;
-      for (int k = b + bwb < nb - 1 ? b + bwb : nb - 1; k > b + BQ_NEAR; --k) {
-        if (tid < 64) vk[tid] = fv[k * 64 + tid];
-        float t[16];
-        bq_load16(gtile(k, b), true, t);
+      for (int k = b + bwb < nb - 1 ? b + bwb : nb - 1; k > b + BQ_NEAR; k -= BQ_FAR) {
+        const int ng = k - b - BQ_NEAR < BQ_FAR ? k - b - BQ_NEAR : BQ_FAR;
+        if (tid < ng * 64) vk[tid >> 6][tid & 63] = fv[(k - (tid >> 6)) * 64 + (tid & 63)];
+        float t[BQ_FAR][16];
+#pragma unroll
+        for (int j = 0; j < BQ_FAR; ++j)
+          if (j < ng) bq_load16(gtile(k - j, b), true, t[j]);
         __syncthreads();
-        s += bq_dot16(t, vk);
+#pragma unroll
+        for (int j = 0; j < BQ_FAR; ++j)
+          if (j < ng) s += bq_dot16(t[j], vk[j]);
         __syncthreads();
       }
 #pragma unroll
