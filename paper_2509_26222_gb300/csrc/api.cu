@@ -371,28 +371,43 @@ rbf_status refresh_center_weights(Ctx* c, cudaStream_t s) {
 
 // The distinct values of one coordinate, ascending.  Mapped terrains have their
 // centers on a lattice, so a hash set finds the few distinct values in one pass
-// (two sorts of 65,536 values took 2.3 ms); scattered centers, with more than
-// DISTINCT_MAX of them, are sorted.
+// (two sorts of 65,536 values took 2.3 ms); centers with more than DISTINCT_MAX of
+// them are sorted, and so are scattered ones as soon as they show: more new values
+// than a lattice not too far from a square has, mostly new ones so far, and
+// neither ascending nor descending as those of a strip of a lattice are.  (3,000
+// scattered centers: 325 us when all were entered first, 304 now, 299 by the
+// sorts alone.)
 static std::vector<double> distinct_values(const std::vector<double>& c, int axis) {
-  constexpr size_t DISTINCT_MAX = 4096, SLOTS = 4 * DISTINCT_MAX;
+  constexpr size_t DISTINCT_MAX = 4096;
   const size_t M = c.size() / 2;
   std::vector<double> u;
+  bool scattered = false;
   if (M > 64) {
-    std::vector<int32_t> slot(SLOTS, -1);
+    const size_t few = 64 + 8 * (size_t)sqrt((double)M);
+    int lg = 9;
+    while (lg < 14 && ((size_t)1 << lg) < 4 * M) ++lg;
+    const size_t mask = ((size_t)1 << lg) - 1;
+    std::vector<int32_t> slot(mask + 1, -1);
+    size_t down = 0;  // new values below the new value before
     for (size_t j = 0; j < M && u.size() <= DISTINCT_MAX; ++j) {
       const double v = c[2 * j + axis] + 0.0;  // -0.0 and 0.0 are one value
       if (!u.empty() && u.back() == v) continue;
       uint64_t bits;
       memcpy(&bits, &v, sizeof(bits));
-      size_t h = (size_t)((bits * 0x9e3779b97f4a7c15ull) >> 50);
-      while (slot[h] >= 0 && u[(size_t)slot[h]] != v) h = (h + 1) & (SLOTS - 1);
+      size_t h = (size_t)((bits * 0x9e3779b97f4a7c15ull) >> (64 - lg));
+      while (slot[h] >= 0 && u[(size_t)slot[h]] != v) h = (h + 1) & mask;
       if (slot[h] < 0) {
         slot[h] = (int32_t)u.size();
+        down += !u.empty() && v < u.back() ? 1 : 0;
         u.push_back(v);
+        if (u.size() > few && 2 * u.size() > j && std::min(down, u.size() - down) > u.size() / 8) {
+          scattered = true;
+          break;
+        }
       }
     }
   }
-  if (M <= 64 || u.size() > DISTINCT_MAX) {
+  if (M <= 64 || scattered || u.size() > DISTINCT_MAX) {
     u.resize(M);
     for (size_t j = 0; j < M; ++j) u[j] = c[2 * j + axis] + 0.0;
   }
