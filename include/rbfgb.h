@@ -295,8 +295,10 @@ enum {
   RBF_STAGE_NEIGHBORS = 0,  /* neighbour lists + active set (bytes: 12 per point) */
   RBF_STAGE_ASSEMBLY = 1,   /* m~ entries, innovation, m~ m~^T rows (flops) */
   RBF_STAGE_BLOCK = 2,      /* leaving/entering centers: Schur complement, stored blocks */
-  RBF_STAGE_PANEL = 3,      /* Cholesky diagonal tiles + panel solves (flops) */
-  RBF_STAGE_TRAILING = 4,   /* Cholesky trailing updates, one interval per launch (flops) */
+  RBF_STAGE_PANEL = 3,      /* Cholesky diagonal tiles + panel solves (flops); the whole factorization where
+                               panels and trailing updates share launches (float64; mixed, dataflow launch) */
+  RBF_STAGE_TRAILING = 4,   /* Cholesky trailing updates that have launches of their own (mixed, launch chain),
+                               one interval per launch (flops) */
   RBF_STAGE_SOLVE = 5,      /* triangular solves and refinement (flops) */
   RBF_STAGE_EVAL = 6,       /* rbf_eval (bytes: 8 in + 12 out per query) */
   RBF_STAGE_SOFTCOST = 7,   /* rbf_soft_cost (bytes: 12 in per point) */

@@ -350,6 +350,15 @@ inline bool not_capturing(cudaStream_t s) {
 constexpr int64_t BW_DENSE = BW_DENSE_CTX;
 rbf_status potrf_lower(Ctx* c, double* A, int64_t n, int64_t lda, int64_t nfactor,
                        bool mixed, cudaStream_t s, int64_t bw = BW_DENSE);
+// Floating-point operations of the first nfactor columns of such a factorization:
+// column j has r_j = min(bw, n - 1 - j) entries below the diagonal, r_j divisions
+// and r_j (r_j + 1) in the update of the rest.
+inline double potrf_work(int64_t n, int64_t nfactor, int64_t bw = BW_DENSE) {
+  auto upto = [](double r) { return r * (r + 1.0) * (2.0 * r + 1.0) / 6.0 + r * (r + 1.0); };  // sum of q^2 + 2 q, q <= r
+  const int64_t full = n - 1 - bw < 0 ? 0 : (n - 1 - bw < nfactor ? n - 1 - bw : nfactor);  // columns with r_j = bw
+  const double w = full > 0 ? (double)full * (double)bw * ((double)bw + 2.0) : 0.0;
+  return nfactor > full ? w + upto((double)(n - 1 - full)) - upto((double)(n - 1 - nfactor)) : w;
+}
 // have_inv: the previous trsm_lower on this context was with the same L
 rbf_status trsm_lower(Ctx* c, const double* L, int64_t n, int64_t ldl, double* B, int64_t m,
                       int64_t ldb, bool transpose, cudaStream_t s, int64_t bw = BW_DENSE, bool have_inv = false);

@@ -267,7 +267,7 @@ rbf_status potrf_lower(Ctx* c, double* A, int64_t n, int64_t lda, int64_t nfacto
   RBF_TRY(dt.ensure(2 * PB * PB * sizeof(double) + (size_t)(steps + 1) * sizeof(int)));
   int* next = reinterpret_cast<int*>(dt.as<double>() + 2 * PB * PB);
   RBF_CUDA(cudaMemsetAsync(next, 0, (size_t)(steps + 1) * sizeof(int), s));
-  StageTimer st(c, RBF_STAGE_PANEL, s, (double)n * n * n / 3.0);
+  StageTimer st(c, RBF_STAGE_PANEL, s, potrf_work(n, nfactor, bw));  // panels and trailing updates share the launches
   const bool early = not_capturing(s);
   PotrfStep P;
   P.A = A;

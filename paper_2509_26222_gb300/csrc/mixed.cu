@@ -605,7 +605,7 @@ static rbf_status potrf_df(Ctx* c, int64_t n, float* W, int64_t ldw, float* Zd, 
   P.wait_xor = c->wait_xor;
   if (ends) P.ends = TwoEnds::make(n, bw);
   void* args[] = {(void*)&P};
-  StageTimer st(c, RBF_STAGE_PANEL, s, (double)n * n * n / 3.0);
+  StageTimer st(c, RBF_STAGE_PANEL, s, potrf_work(n, n, bw));
   RBF_CUDA(cooperative_launch(kern, dim3((unsigned)grid), dim3(DF_THREADS), args, smem, s));
   return RBF_OK;
 }
