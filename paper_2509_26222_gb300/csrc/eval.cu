@@ -581,16 +581,24 @@ __global__ void __launch_bounds__(SC_MAX_THREADS) k_soft_cost(EvalParams P, cons
   sc_block_sums<NV>(acc, partials);
 }
 
-// Sum over the blocks of value (warp index) of the partial rows, in lane 0:
-// lanes stride over the blocks, so that the loads of a value are in flight
-// together (one lane per value took 15 us for 256 blocks).
-__device__ __forceinline__ double sc_total(const double* __restrict__ partials, int nblk, int stride, int k) {
-  const int lane = threadIdx.x & 31;
-  double v = 0;
-  for (int b = lane; b < nblk; b += 32) v += partials[(int64_t)b * stride + k];
+// Sums over the blocks of the values k0, k0 + step, .. (N of them) of the partial
+// rows, by a warp: lanes stride over the blocks, so that the loads of a value are in
+// flight together (one lane per value took 15 us for 256 blocks).
+template <int N>
+__device__ __forceinline__ void sc_totals(const double* __restrict__ partials, int nblk, int stride, int k0, int step,
+                                          double (&v)[N]) {
+  for (int b = threadIdx.x & 31; b < nblk; b += 32)
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+    for (int q = 0; q < N; ++q) v[q] += partials[(int64_t)b * stride + k0 + q * step];
+#pragma unroll
+  for (int q = 0; q < N; ++q)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+}
+__device__ __forceinline__ double sc_total(const double* __restrict__ partials, int nblk, int stride, int k) {
+  double v[1] = {0.0};
+  sc_totals<1>(partials, nblk, stride, k, 0, v);
+  return v[0];
 }
 
 // out[0] = cost, out[1..6] = gradient, out[7..27] = A (when nv = 28); the
@@ -955,22 +963,27 @@ extern "C" rbf_status rbf_soft_cost_normal(rbf_ctx* c, const double* R, const do
 }
 
 // The Levenberg-Marquardt step of the pose from the partial sums of
-// soft_cost_partials<28>: one warp per value takes the totals v28 (the layout
+// soft_cost_partials<28>: a warp per two values takes the totals v28 (the layout
 // of rbf_soft_cost_normal), then one thread forms B = A + mu diag(A), factors
 // it (Cholesky, float64), solves B delta = -g and applies R Exp(delta_theta)
 // (Rodrigues' formula), t + delta_t.  The serial part is a chain of float64
 // square roots, divisions and sines: the loops are unrolled so that the
-// matrices stay in registers, and each pivot is inverted once (16.3 us with
-// the totals; 17.8 us after a reduction launch of 3.4 us with indexed local
-// arrays and a division per entry).
-__global__ void __launch_bounds__(32 * SC_NORMAL) k_lm_solve(const double* __restrict__ partials, int nblk, double mu, Pose T,
+// matrices stay in registers, which two values a warp leave enough of (a warp a
+// value caps them at 72 a thread, with spills), and each pivot is inverted once
+// (whole step of 65,536 points 51.3 us, 52.5 with the spills; the kernel with them
+// 16.3 us with the totals, and 17.8 after a reduction launch
+// of 3.4 us, with indexed local arrays and a division per entry).
+constexpr int LM_WARPS = SC_NORMAL / 2;
+__global__ void __launch_bounds__(32 * LM_WARPS) k_lm_solve(const double* __restrict__ partials, int nblk, double mu, Pose T,
                                                   double* __restrict__ out) {
   __shared__ double v28[SC_NORMAL];
   {
     const int k = threadIdx.x >> 5;
-    if (k < SC_NORMAL) {
-      const double v = sc_total(partials, nblk, sc_pad(SC_NORMAL), k);
-      if ((threadIdx.x & 31) == 0) v28[k] = v;
+    double v[2] = {0.0, 0.0};
+    sc_totals<2>(partials, nblk, sc_pad(SC_NORMAL), k, LM_WARPS, v);
+    if ((threadIdx.x & 31) == 0) {
+      v28[k] = v[0];
+      v28[k + LM_WARPS] = v[1];
     }
   }
   __syncthreads();
@@ -1071,7 +1084,7 @@ extern "C" rbf_status rbf_lm_step(rbf_ctx* c, const double* R, const double* t, 
     StageTimer st(x, RBF_STAGE_SOFTCOST, s, 12.0 * (double)n);
     RBF_TRY(soft_cost_partials(x, T, pts, n, nullptr, s, true, &pp, &nb));
   }
-  { k_lm_solve<<<1, 32 * SC_NORMAL, 0, s>>>(pp, nb, mu, T, out20); ::rbf::note_launch(); }
+  { k_lm_solve<<<1, 32 * LM_WARPS, 0, s>>>(pp, nb, mu, T, out20); ::rbf::note_launch(); }
   RBF_CUDA(cudaGetLastError());
   return RBF_OK;
 }
