@@ -17,7 +17,6 @@
 namespace rbf {
 namespace {
 
-// nonzeros per row (one warp per row)
 // nonzeros per row (one warp per row) and the half-bandwidth max |i - j|
 // over the nonzero entries (atomicMax into *bw)
 __global__ void __launch_bounds__(256) k_csr_count(const double* __restrict__ H, int64_t n, int64_t ld, int64_t band,

@@ -125,7 +125,8 @@ __global__ void __launch_bounds__(128) k_syrk_tc(float* __restrict__ Cm, int64_t
 
   // epilogue: warp w owns TMEM lanes (rows) 32 w .. 32 w + 31.  A thread puts its
   // row, negated, where the operands were (they are read) and adds it to C with
-  // one bulk reduction: C never comes to the SM, and C + (-x) is C - x to the bit.
+  // one bulk reduction: C never comes to the SM, and C + (-x) is C - x to the bit
+  // (the reduction flushes subnormal values to zero, 1e-38 against entries of 1).
   const int64_t row = i0 + warp * 32 + lane;
   const int ncol = (int)(m - j0 < TILE ? m - j0 : TILE), nb4 = ncol & ~3;
   if (done) {

@@ -1227,12 +1227,10 @@ extern "C" rbf_status rbf_update(rbf_ctx* cx, const float* pts, int64_t n, doubl
     { k_diag_add<<<nblk(an), 256, 0, s>>>(Hn.as<double>(), ld, an, c->diag_shift); ::rbf::note_launch(); }
     RBF_CUDA(cudaGetLastError());
   }
-  // Until a center has left some block there is no Schur-complement fill and
-  // H' has the band structure of m~ m~^T: read its half-bandwidth then (a first
-  // update has it from its lists already), and
-  // skip the zero blocks outside the band in the factorization and solves.
-  // Otherwise the compressed rows of H' (needed from the first residual of
-  // the solve on) are built on a side stream beside the factorization.
+  // Until a center has left some block there is no Schur-complement fill and H'
+  // has the band structure of m~ m~^T: its half-bandwidth (a first update has it
+  // from its lists already) lets the factorization and the solves skip the zero
+  // blocks outside.
   const bool band_probe = !c->pg_on && d == 0;
   // Once a center has left, H' carries Schur fill and soon holds about a^2
   // nonzeros: its residuals then read the dense H' (8 bytes an entry against
@@ -1242,9 +1240,10 @@ extern "C" rbf_status rbf_update(rbf_ctx* cx, const float* pts, int64_t n, doubl
     else c->Hs_next.valid = false;
   }
   if (band_probe) {
-    if (list_band) ;
-    else if (mixed && c->Hs_next.valid) RBF_TRY(csr_bandwidth(c, an, &bw, s));
-    else RBF_TRY(dense_bandwidth(c, Hn.as<double>(), ld, an, &bw, s));
+    if (!list_band) {
+      if (mixed && c->Hs_next.valid) RBF_TRY(csr_bandwidth(c, an, &bw, s));
+      else RBF_TRY(dense_bandwidth(c, Hn.as<double>(), ld, an, &bw, s));
+    }
     if (3 * bw >= an) bw = BW_DENSE;
   }
 
