@@ -229,7 +229,8 @@ __device__ __forceinline__ BqM bq_fixed(FF m) {
   BqM r;
   r.k = k;
   r.q = __float2ull_rn(m.hi * f) + (unsigned long long)__float2ll_rn(m.lo * f);
-  r.q52 = k < 116 ? ((r.q >> (k - 53)) + 1ull) >> 1 : 0ull;
+  constexpr float f52 = 4503599627370496.f;
+  r.q52 = __float2ull_rn(m.hi * f52) + (unsigned long long)__float2ll_rn(m.lo * f52);
   return r;
 }
 __device__ __forceinline__ BqM bq_fixed(double m) {
@@ -619,10 +620,14 @@ constexpr int BQ_FAR = 4;   // tiles farther off whose loads are in flight toget
 // memory.  Tiles farther off follow in groups.  256 patches, nb up to 64: three
 // sweeps 2.14 -> 1.98 ms.  Batch of four patches of 128 x 128 (12 tiles): 21.5 ms
 // with the far tiles one by one, 20.2 in threes, 19.5 in fours (and 36 bytes of spills).
+// FAR (patches whose band has more than BQ_NEAR tiles) is an instance of its own:
+// the groups take the kernel from 161 to 255 registers, and batches without them
+// were 1.5 % slower.
+template <bool FAR>
 __global__ void __launch_bounds__(256) k_bq_solve(const BqPatch* __restrict__ P, int np, const float* __restrict__ Wt,
                                                   const float* __restrict__ Zd, const double* __restrict__ r,
                                                   float* __restrict__ f, double* __restrict__ x, int* __restrict__ counter) {
-  __shared__ float acc[64], vk[BQ_FAR][64], ring[8][64];  // block k of the solution in ring[k % 8]
+  __shared__ float acc[64], vk[FAR ? BQ_FAR : 1][64], ring[8][64];  // block k of the solution in ring[k % 8]
   __shared__ int cur;
   const int tid = threadIdx.x, row = tid >> 2, part = tid & 3;
   for (;;) {
@@ -651,7 +656,7 @@ __global__ void __launch_bounds__(256) k_bq_solve(const BqPatch* __restrict__ P,
     for (int b = 0; b < nb; ++b) {
       const float rb = part == 0 ? (float)rv[b * 64 + row] : 0.f;
       float s = 0.f;
-      for (int k = b - bwb > 0 ? b - bwb : 0; k < b - BQ_NEAR; k += BQ_FAR) {
+      for (int k = b - bwb > 0 ? b - bwb : 0; FAR && k < b - BQ_NEAR; k += BQ_FAR) {
         const int ng = b - BQ_NEAR - k < BQ_FAR ? b - BQ_NEAR - k : BQ_FAR;
         if (tid < ng * 64) vk[tid >> 6][tid & 63] = fv[k * 64 + tid];
         float t[BQ_FAR][16];
@@ -693,7 +698,7 @@ __global__ void __launch_bounds__(256) k_bq_solve(const BqPatch* __restrict__ P,
     for (int b = nb - 1; b >= 0; --b) {
       const float yb = part == 0 ? fv[b * 64 + row] : 0.f;
       float s = 0.f;
-      for (int k = b + bwb < nb - 1 ? b + bwb : nb - 1; k > b + BQ_NEAR; k -= BQ_FAR) {
+      for (int k = b + bwb < nb - 1 ? b + bwb : nb - 1; FAR && k > b + BQ_NEAR; k -= BQ_FAR) {
         const int ng = k - b - BQ_NEAR < BQ_FAR ? k - b - BQ_NEAR : BQ_FAR;
         if (tid < ng * 64) vk[tid >> 6][tid & 63] = fv[(k - (tid >> 6)) * 64 + (tid & 63)];
         float t[BQ_FAR][16];
@@ -1076,6 +1081,9 @@ static rbf_status bq_enqueue(Ctx* c, BqState* S, BqPlan& L, const BqGeom& G, cud
     const int sweeps = std::min(c->refine_sweeps > 0 ? c->refine_sweeps : 3, 16);
     RBF_CUDA(cudaMemsetAsync(L.x.p, 0, (size_t)L.nvec * sizeof(double), s));
     RBF_CUDA(cudaMemcpyAsync(L.r.p, L.u.p, (size_t)L.nvec * sizeof(double), cudaMemcpyDeviceToDevice, s));
+    bool far = false;
+    for (const BqPatch& B : L.patches) far |= B.bwb > BQ_NEAR;
+    auto solve = far ? k_bq_solve<true> : k_bq_solve<false>;
     for (int it = 0; it < sweeps; ++it) {
       if (it > 0) {
         { k_bq_tile_products<<<(unsigned)L.ntiles, 256, 0, s>>>(dP, np, reinterpret_cast<const double*>(L.tiles64.p),
@@ -1085,9 +1093,9 @@ static rbf_status bq_enqueue(Ctx* c, BqState* S, BqPlan& L, const BqGeom& G, cud
                                                           L.r.as<double>()); ::rbf::note_launch(); }
         RBF_CUDA(cudaGetLastError());
       }
-      { k_bq_solve<<<(unsigned)std::min(np, 4 * sms), 256, 0, s>>>(dP, np, L.tiles32.as<float>(), L.zd.as<float>(),
-                                                               L.r.as<double>(), L.f.as<float>(), L.x.as<double>(),
-                                                               cnt + 1 + it); ::rbf::note_launch(); }
+      { solve<<<(unsigned)std::min(np, 4 * sms), 256, 0, s>>>(dP, np, L.tiles32.as<float>(), L.zd.as<float>(),
+                                                              L.r.as<double>(), L.f.as<float>(), L.x.as<double>(),
+                                                              cnt + 1 + it); ::rbf::note_launch(); }
       RBF_CUDA(cudaGetLastError());
     }
     { k_bq_store_w<<<bq_blocks(L.nvec), 256, 0, s>>>(dP, np, L.nvec, L.x.as<double>(), L.f.as<float>()); ::rbf::note_launch(); }
