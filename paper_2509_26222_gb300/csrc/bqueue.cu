@@ -179,22 +179,29 @@ __device__ __forceinline__ void bq_add_mz(unsigned long long* u2, unsigned long 
   const unsigned bits = __float_as_uint(z);
   const int ex = (bits >> 23) & 255;
   const unsigned long long mant = (bits & 0x7fffffu) | (ex ? 0x800000u : 0u);
-  unsigned long long lo = q * mant, hi = __umul64hi(q, mant);
-  const int sh = (ex ? ex : 1) - 86 - k;  // z = mant 2^(ex - 150)
-  if (sh >= 0) {
-    if (sh >= 64) {
-      hi = sh < 128 ? lo << (sh - 64) : 0ull;
-      lo = 0ull;
-    } else if (sh > 0) {
-      hi = (hi << sh) | (lo >> (64 - sh));
-      lo <<= sh;
-    }
-  } else if (sh > -64) {
-    lo = (lo >> -sh) | (hi << (64 + sh));
-    hi >>= -sh;
+  const int r = 86 + k - (ex ? ex : 1);  // units of 2^-64 from the product: z = mant 2^(ex - 150)
+  unsigned long long lo, hi = 0ull;
+  if ((unsigned)(r - 24) < 40u) {
+    lo = __umul64hi(q, mant << (64 - r));  // (q mant) >> r
   } else {
-    lo = sh > -128 ? hi >> (-sh - 64) : 0ull;
-    hi = 0ull;
+    lo = q * mant;
+    hi = __umul64hi(q, mant);
+    const int sh = -r;
+    if (sh >= 0) {
+      if (sh >= 64) {
+        hi = sh < 128 ? lo << (sh - 64) : 0ull;
+        lo = 0ull;
+      } else if (sh > 0) {
+        hi = (hi << sh) | (lo >> (64 - sh));
+        lo <<= sh;
+      }
+    } else if (sh > -64) {
+      lo = (lo >> -sh) | (hi << (64 + sh));
+      hi >>= -sh;
+    } else {
+      lo = sh > -128 ? hi >> (-sh - 64) : 0ull;
+      hi = 0ull;
+    }
   }
   if (bits >> 31) {
     lo = ~lo + 1ull;
