@@ -189,8 +189,8 @@ __global__ void __launch_bounds__(256) k_trtri_level(int kind, int64_t b, int64_
 // two.  B comes as rows of K, so a thread splits two neighbouring rows and stores
 // pairs, which makes B K-major.  At half-size 512 this kernel takes as long as the
 // float32 tiles (48 + 52 us and 41 + 58 for the two products): the line is at 1024.
-// Whole inverse, float32 tiles and now: n = 1,810 225 / 166 us, 2,500 517 / 269,
-// 3,750 936 / 443, 5,000 1,959 / 922.
+// Whole inverse, float32 tiles and now: n = 1,810 225 / 164 us, 2,500 517 / 266,
+// 3,750 936 / 425, 5,000 1,959 / 899.
 //
 // No further from 64 bits than float32 multiply-adds (0.77 to 1.00 times, block by
 // block), because
@@ -201,13 +201,15 @@ __global__ void __launch_bounds__(256) k_trtri_level(int kind, int64_t b, int64_
 //    added before the one rounding (rounded apart and added in memory: up to 1.03);
 //  * the first product, whose errors the second one amplifies, takes all products
 //    but l l, the second one h h, h m, h l and m m (six for both: up to 1.0004).
-// The three cost 6 to 10 % of the inverse.
+// (One accumulator, six products and sums in memory: 160, 258, 434 and 950 us.)
 constexpr int TT_MIN = 1024;
 constexpr int TT_K = 64;
 constexpr int TT_SLICE = 128 * TT_K * 2;             // bytes of a 128 x 64 bf16 slice
-constexpr int TT_SMEM = 6 * TT_SLICE + 1024;
 constexpr uint32_t TT_COLS = 256;
-constexpr int TT_ROW = 128 * 4 + 16;                 // bytes of a staged output row (padded over the banks)
+constexpr int TT_ROW = 128 * 4 + 32;                 // bytes of a staged output row (padded over the banks)
+constexpr int TT_TURN = 32 * 36 * 4;                 // bytes of a warp's 32 x 32 floats on their way to the peer
+constexpr int TT_SMEM = 128 * TT_ROW + 8 * TT_TURN + 1024;  // the operands (6 slices) lie in the same place
+static_assert(128 * TT_ROW + 8 * TT_TURN >= 6 * TT_SLICE, "operands");
 
 // x and y as three bfloat16 each (24 bits, every slice rounded to nearest; a NaN
 // stays one), slice t of x in the low and of y in the high half of q[t].  (With the
@@ -389,12 +391,25 @@ __global__ void __launch_bounds__(256, 2) k_trtri_tc(int kind, int64_t b, int64_
     tc::cluster_arrive();
     load(64 * (int)(rank ^ 1) + 32 * q);
     tc::cluster_wait();  // both have read their operands
-    const uint32_t to = tc::cluster_addr(tc::smem_u32(sm + lr * TT_ROW) + 128u * q, rank ^ 1);
+    // turned in shared memory, so that eight lanes store the 128 bytes of a row (with
+    // a row a lane, in pieces of 16 bytes, the inverse of 3,750 rows took 441 us)
+    const uint32_t to = tc::cluster_addr(tc::smem_u32(sm), rank ^ 1);
+    float* st = reinterpret_cast<float*>(sm + 128 * TT_ROW + warp * TT_TURN);
+    auto give = [&](const float (&x)[32], uint32_t off) {
 #pragma unroll
-    for (int e = 0; e < 32; e += 4) {
-      tc::cluster_store4(to + 4 * e, v[e], v[e + 1], v[e + 2], v[e + 3]);
-      tc::cluster_store4(to + 256 + 4 * e, v2[e], v2[e + 1], v2[e + 2], v2[e + 3]);
-    }
+      for (int e = 0; e < 32; e += 4)
+        *reinterpret_cast<float4*>(st + lane * 36 + e) = make_float4(x[e], x[e + 1], x[e + 2], x[e + 3]);
+      __syncwarp();
+#pragma unroll
+      for (int t = 0; t < 32; t += 4) {
+        const int r = t + (lane >> 3);
+        const float4 y = *reinterpret_cast<const float4*>(st + r * 36 + 4 * (lane & 7));
+        tc::cluster_store4(to + (uint32_t)((32 * (warp & 3) + r) * TT_ROW) + off + 16u * (lane & 7), y.x, y.y, y.z, y.w);
+      }
+      __syncwarp();
+    };
+    give(v, 128u * q);
+    give(v2, 256u + 128u * q);
     tc::cluster_arrive();
     load(64 * (int)rank + 32 * q);
     tc::cluster_wait();
