@@ -11,7 +11,7 @@
 //               chunks of ch x ch lattice nodes (three launches);
 //  2. Gram      persistent CTAs pull chunks from a counter; a CTA adds the
 //               products m_{i,a} m_{i,b} and m_{i,a} z_i of the chunk's
-//               points exactly (fixed-point integers, as the main update)
+//               points in any order to the same bits (fixed-point integers)
 //               into a window of the band in shared memory, then flushes
 //               the nonzero sums to the patch's band tiles with one global
 //               atomic each;

@@ -200,7 +200,8 @@ __global__ void __launch_bounds__(256) k_trtri_level(int kind, int64_t b, int64_
 //    each, they are a cluster and swap halves of their accumulators, which are
 //    added before the one rounding (rounded apart and added in memory: up to 1.03);
 //  * the first product, whose errors the second one amplifies, takes all products
-//    but l l, the second one h h, h m, h l and m m (six for both: up to 1.0004).
+//    but l l, the second one h h, h m, m h, h l, l h and m m (these six for both:
+//    up to 1.0004).
 // (One accumulator, six products and sums in memory: 160, 258, 434 and 950 us.)
 constexpr int TT_MIN = 1024;
 constexpr int TT_K = 64;
